@@ -1,0 +1,60 @@
+"""The CTA-pair tensor-core X-engine (129 to 256 inputs): tile, stage and team
+edges, ragged last tiles, adding launches and the fused beam, bit-exact against
+the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1501_05992_gb300 import corr
+
+from _gpu import path_available
+
+pytestmark = pytest.mark.gpu
+
+
+# inputs around the two tiles' edges (one input, half a tile and all but one in
+# the second); samples around a 64-sample stage and the four teams' turns; more
+# channels than CTA pairs where a pair must take several items
+@pytest.mark.parametrize("N,F,T", [(129, 2, 65), (144, 3, 64), (176, 1, 1), (192, 2, 63), (193, 90, 130), (208, 3, 257),
+                                   (250, 2, 320), (255, 1, 191), (256, 160, 300), (256, 1, 4100)])
+@pytest.mark.parametrize("zero_invalid", [False, True])
+def test_pair_blocks_exact(N, F, T, zero_invalid):
+    if not path_available("tc_fp8", N):
+        pytest.skip("tc_fp8 unsupported")
+    volt = np.random.default_rng(N + F + T).integers(0, 256, (T, F, N), dtype=np.uint8)
+    c = corr.Correlator(N, F, 2 * T, path="tc_fp8", zero_invalid=zero_invalid)
+    d = torch.from_numpy(volt).cuda()
+    tri, beam = c.integrate_beam(d, 1)
+    whole = c.integrate(d)
+    h = T // 3
+    if h:
+        c.accumulate(d[:h])
+    c.accumulate(d[h:])
+    c.accumulate(d)
+    acc = c.dump()
+    c.sync()
+    c.close()
+    vis = oracle.xmac(volt, zero_invalid)
+    assert np.array_equal(whole.cpu().numpy(), oracle.to_int32(vis))
+    assert np.array_equal(tri.cpu().numpy(), oracle.to_int32(vis))
+    assert np.array_equal(acc.cpu().numpy(), oracle.to_int32(2 * vis))
+    assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
+
+
+@pytest.mark.parametrize("byte", [0x77, 0x88, 0x80, 0x08, 0x87, 0x78])
+def test_pair_extreme_sums_exact(byte):
+    """Constant samples of the largest codes over 33000 samples: the largest FP32
+    partial sums a launch of 32768 samples can reach, and its split."""
+    if not path_available("tc_fp8", 256):
+        pytest.skip("tc_fp8 unsupported")
+    N, F, T = 256, 1, 33000
+    volt = np.full((T, F, N), byte, np.uint8)
+    volt[:, :, 128:] = (byte >> 4) | ((byte << 4) & 0xFF)
+    c = corr.Correlator(N, F, T, path="tc_fp8")
+    got = c.integrate(torch.from_numpy(volt).cuda())
+    c.sync()
+    c.close()
+    # every sample is the same: T times the product of one
+    want = oracle.xmac(volt[:1]) * T
+    assert np.array_equal(got.cpu().numpy(), oracle.to_int32(want))
