@@ -100,12 +100,13 @@ int corr_destroy(corr_ctx *ctx);
 
 /* Select the implementation.  CORR_E_UNSUPPORTED if the path cannot run on
  * this device (CORR_PATH_TC_FP8 needs an sm_103 device).  The tensor-core
- * path reads the voltage rows through TMA, which needs rows on 16-byte
- * boundaries: with n_inputs % 16 != 0 each call's samples are first copied
- * into rows of round_up(n_inputs, 16) bytes in the workspace (up to 4 GiB:
- * a whole integration where it fits, else chunks of a multiple of 64
- * samples), and in a batch such arrays are
- * correlated in launches of their own.  AUTO picks the tensor-core path from
+ * path reads the rows of 129 to 256 inputs (tile 0 or 256, corr_set_tile) as
+ * they are, on any byte boundary; other rows come through TMA, which needs
+ * them on 16-byte boundaries: with n_inputs % 16 != 0 each call's samples are
+ * first copied into rows of round_up(n_inputs, 16) bytes in the workspace (up
+ * to 4 GiB: a whole integration where it fits, else chunks of a multiple of 64
+ * samples).  In a batch, arrays with n_inputs % 16 != 0 are correlated in
+ * launches of their own.  AUTO picks the tensor-core path from
  * 64 inputs on.  Valid only between integrations (corr_samples() == 0), else
  * CORR_E_STATE.  The default is CORR_PATH_AUTO. */
 int corr_set_path(corr_ctx *ctx, int path);
@@ -115,9 +116,11 @@ int corr_set_path(corr_ctx *ctx, int path);
  * item one 128 x 128 tile pair (one TMEM accumulator each, so an item's
  * epilogue overlaps the next item's MMAs); 256 = pair items, a diagonal tile
  * and the tile left of it as one 256-row column of the triangle (one
- * conversion of the shared tile feeds two accumulators).  0 chooses by shape:
- * 32 when n_inputs <= 32 on the CUDA-core path; pair items from 64 stages
- * of 64 samples per launch on the tcgen05 path.  A value that does not apply
+ * conversion of the shared tile feeds two accumulators), and for 129 to 256
+ * inputs the whole 256 x 256 block of a channel as one item of a pair of SMs.
+ * 0 chooses by shape: 32 when n_inputs <= 32 on the CUDA-core path; on the
+ * tcgen05 path the 256 x 256 block for 129 to 256 inputs, else pair items from
+ * 64 stages of 64 samples per launch.  A value that does not apply
  * to the context's path is ignored by it.  Any other value: CORR_E_ARG.  Only
  * between integrations (CORR_E_STATE). */
 int corr_set_tile(corr_ctx *ctx, int tile);

@@ -213,9 +213,10 @@ int accumulate_to(corr_ctx *c, const uint8_t *volt, int nt, int32_t *target, boo
     cudaError_t e = cudaSuccess;
     const size_t row = size_t(c->f) * size_t(c->n);
     if (path == CORR_PATH_TC_FP8) {
-        // rows of n % 16 != 0 inputs go through a padded copy, chunk by chunk
-        const int pad_t = tc_pad_samples(c->n, c->f, c->t_max);
-        if (!pad_t && (reinterpret_cast<uintptr_t>(volt) & 15) != 0) return CORR_E_ARG;
+        // rows of n % 16 != 0 inputs go through a padded copy, chunk by chunk, except
+        // where the kernel reads them as they are
+        if (c->n % 16 == 0 && (reinterpret_cast<uintptr_t>(volt) & 15) != 0) return CORR_E_ARG;
+        const int pad_t = tc_any_rows(c->n, tc_items(c)) ? 0 : tc_pad_samples(c->n, c->f, c->t_max);
         const int step = pad_t ? (pad_t < kTcMaxSamples ? pad_t : kTcMaxSamples) : kTcMaxSamples;
         for (int t0 = 0; t0 < nt; t0 += step) {
             const int ntc = nt - t0 < step ? nt - t0 : step;

@@ -97,12 +97,15 @@ struct TcArray {
     int n_chan, n, nt;
     bool zero_invalid, fresh;
     TcItems items = TcItems::kAuto;
-    int ld = 0;            // row stride in bytes, a multiple of 16 (0: n)
+    int ld = 0;            // row stride in bytes (0: n); a multiple of 16 unless tc_any_rows()
     // incoherent beam of the same samples, added into beam[(beam_t0 + t) /
     // beam_avg][n_chan] (zeroed by the caller); NULL for none
     int32_t *beam = nullptr;
     int beam_avg = 1, beam_t0 = 0;
 };
+// Whether an array of n inputs runs on the CTA-pair kernel (xeng_pair.cu), which
+// takes rows on any byte boundary.
+bool tc_any_rows(int n, TcItems items);
 // Samples per padded copy for the tensor-core path when n % 16 != 0: the
 // whole integration if it fits kTcPadCap bytes, else chunks of a multiple
 // of 64 samples.

@@ -36,6 +36,13 @@
 // shared-memory pipe is 70 % busy, the tensor pipe 63 %, the ALU pipe 50 %.  Short
 // launches (64 samples) are bound by the epilogue's exchange and stores.
 //
+// Rows on any byte boundary (input counts that are no multiple of 16) are read
+// as they are, as aligned words: 250 inputs x 760 channels x 5000 samples 0.47 ms
+// (0.54 ms with invalid samples zeroed) against 0.33 ms for 256 inputs, where a
+// copy into padded rows first took 0.41 ms by itself.  (A lane per word of a row
+// instead of four words of a 16-byte chunk: 0.53 and 0.60 ms, for its 4-byte
+// plane stores and two shuffles per word.)
+//
 // Roles per CTA (persistent; items are strided over the pairs):
 //   warps 0-7    epilogue, two warps per quarter of the accumulator's lanes
 //   warps 8-23   converters: four teams of four warps (one per scheduler) that
@@ -101,7 +108,7 @@ struct ArrayParams {
     long long row_t;          // bytes from one sample of a channel to the next
     int ld;                   // bytes from one channel to the next
     int32_t *acc;
-    int n, n_blocks, nt, n_stages, item_begin, fresh;
+    int n, n_chan, n_blocks, nt, n_stages, item_begin, fresh;
     int32_t *beam;
     int beam_ld, beam_avg, beam_t0;
 };
@@ -112,7 +119,7 @@ struct Params {
     DeviceStatus *status;
     long long wait_limit;
     int inject_stall;
-    uint32_t one, minus_one, sixteen;   // multipliers of imad()
+    uint32_t one, minus_one, fifteen, sixteen;   // multipliers of imad()
 };
 
 struct Item {
@@ -232,15 +239,6 @@ __device__ __forceinline__ void commit_own(uint32_t bar)
     asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
-// The four samples of w with code 8 in either part set to zero.
-__device__ __forceinline__ uint32_t zero_invalid4(uint32_t w)
-{
-    const uint32_t x = w ^ 0x88888888u;           // a nibble code of 8 becomes 0
-    uint32_t t = x | (x >> 1);
-    t |= t >> 2;                                  // bit 0 of each nibble: the code was not 8
-    return w & ((t & (t >> 4) & 0x01010101u) * 0xFFu);
-}
-
 // a * b + c as one multiply-add (the FMA pipe).  b is a kernel parameter, so that
 // the compiler cannot turn it back into an add or a shift: the ALU pipe takes one
 // warp instruction per two cycles, the FMA pipe beside it another, and this
@@ -256,17 +254,28 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c)
 // Planes of the four packed samples of w (real part in the high nibbles): q =
 // r - m, r and 2 m as E4M3 sign and magnitude.  ur, um are v + 8 and |v| the
 // byte-wise distance from the offset; the signs of r and m are their nibbles'
-// top bits and that of q is the borrow of ur - um + 128.
-__device__ __forceinline__ void planes4(uint32_t w, uint32_t one, uint32_t minus_one, uint32_t sixteen, uint32_t &Q,
-                                        uint32_t &R, uint32_t &M)
+// top bits and that of q is the borrow of ur - um + 128.  With kZeroInvalid a
+// sample with code 8 (u = 0) in either part becomes 0 + 0i (u = 8; the signs of
+// its zeros do not matter), in w too.
+template <bool kZeroInvalid>
+__device__ __forceinline__ void planes4(uint32_t &w, const Params &p, uint32_t &Q, uint32_t &R, uint32_t &M)
 {
     const uint32_t x = w ^ 0x88888888u;
-    const uint32_t um = x & 0x0F0F0F0Fu;
-    const uint32_t ur = (x >> 4) & 0x0F0F0F0Fu;
-    const uint32_t t = imad(um, minus_one, imad(ur, one, 0x80808080u));
+    uint32_t um = x & 0x0F0F0F0Fu;
+    uint32_t ur = (x >> 4) & 0x0F0F0F0Fu;
+    const uint32_t sign_r = w & 0x80808080u, w16 = imad(w, p.sixteen, 0u);
+    if (kZeroInvalid) {
+        // bit 4 of u + 15: u != 0
+        const uint32_t ok = imad(ur, p.one, 0x0F0F0F0Fu) & imad(um, p.one, 0x0F0F0F0Fu) & 0x10101010u;
+        const uint32_t low = imad(ok >> 4, p.fifteen, 0u);
+        ur = (ur & low) | (0x08080808u & ~low);
+        um = (um & low) | (0x08080808u & ~low);
+        w &= imad(low, p.sixteen, low);
+    }
+    const uint32_t t = imad(um, p.minus_one, imad(ur, p.one, 0x80808080u));
     Q = __vabsdiffu4(ur, um) | (~t & 0x80808080u);
-    R = __vabsdiffu4(ur, 0x08080808u) | (w & 0x80808080u);
-    M = __vabsdiffu4(imad(um, one, um), 0x10101010u) | (imad(w, sixteen, 0u) & 0x80808080u);
+    R = __vabsdiffu4(ur, 0x08080808u) | sign_r;
+    M = __vabsdiffu4(imad(um, p.one, um), 0x10101010u) | (w16 & 0x80808080u);
 }
 
 __device__ __forceinline__ uint4 load16(const uint8_t *a)
@@ -287,7 +296,7 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&r)[16])
         : "r"(taddr));
 }
 
-template <bool kZeroInvalid, bool kBeam>
+template <bool kAligned, bool kZeroInvalid, bool kBeam>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 xeng_pair_kernel(const __grid_constant__ Params p)
 {
@@ -395,6 +404,12 @@ xeng_pair_kernel(const __grid_constant__ Params p)
         // Team t converts the stages g (counted over all items of this CTA) with
         // g % kTeams == t, so each warp meets the barriers once per kTeams stages.
         // A thread owns chunk column c (16 inputs) of rows (samples) q + k kRowStep.
+        // kAligned: rows start on 16-byte boundaries, a chunk is one load.  Otherwise a
+        // chunk is the four aligned words from the one that holds its first byte; the
+        // bytes past them come from the first word of the next lane's chunk, for the
+        // row's last chunk (c = 7) from one more word that lane r of the warp loads for
+        // the warp's r-th row.  A row's offset from a word boundary is the same for all
+        // of a thread's rows (16 samples apart).
         const int ci = warp - kFirstConvWarp;
         const int u = (ci % kTeamWarps) * 32 + lane;
         const int c = u & 7, q = u >> 3;
@@ -407,19 +422,41 @@ xeng_pair_kernel(const __grid_constant__ Params p)
         const uint8_t *ptr = nullptr;
         int32_t *beam = nullptr;
         int beam_avg = 1, beam_ld = 0, t_beam = 0;
+        // rows on any byte: this thread's inputs from its chunk on, its rows' offset from
+        // a word boundary, whether the item has such offsets; the extra word's address and
+        // the number of samples it is there for; the array's bytes and whether the item
+        // has words that reach over their ends (its first and last channels)
+        int left = kTile, sh = 0, x_rows = 0;
+        bool skew = false, edge = false;
+        const uint8_t *x_ptr = nullptr, *lo = nullptr, *hi = nullptr;
         auto enter = [&] {                     // stage s of `item`, or of a later one past its end
             while (item < p.n_items) {
                 const Item it = decode_item(p, item);
                 const ArrayParams &A = p.a[it.a];
                 n_stages = A.n_stages;
                 if (s < n_stages) {
-                    const int x = it.base + rank * kTile + c * 16;
+                    const int tile = it.base + rank * kTile;
+                    const uint8_t *const first = A.volt + (long long)it.f * A.ld + tile;
                     row_t = A.row_t;
+                    left = A.n - tile - c * 16;
+                    ptr = first + c * 16 + (long long)(s * kTc + q) * row_t;
+                    if (!kAligned) {
+                        sh = int(reinterpret_cast<uintptr_t>(ptr) & 3);
+                        ptr -= sh;
+                        skew = ((reinterpret_cast<uintptr_t>(first) | uintptr_t(row_t)) & 3) != 0;
+                        const int xt = s * kTc + (q & ~3) + (lane & 3) + (lane >> 2) * kRowStep;
+                        x_ptr = first + kTile + (long long)xt * row_t;
+                        const int xs = int(reinterpret_cast<uintptr_t>(x_ptr) & 3);
+                        x_ptr -= xs;
+                        x_rows = lane < 4 * kUnits && xs && A.n - tile - kTile + xs > 0 ? A.nt - xt : 0;
+                        edge = it.f == 0 || it.f == A.n_chan - 1;
+                        lo = A.volt;
+                        hi = A.volt + (long long)A.nt * row_t;
+                    }
                     // rows of this thread with a sample (none for a chunk past the inputs)
-                    rows = x < A.n ? A.nt - q - s * kTc : 0;
+                    rows = left + sh > 0 ? A.nt - q - s * kTc : 0;
                     // stages of this item from s on whose loads need no bounds
-                    whole = it.base + (rank + 1) * kTile <= A.n ? A.nt / kTc - s : 0;
-                    ptr = A.volt + (long long)it.f * A.ld + x + (long long)(s * kTc + q) * row_t;
+                    whole = tile + kTile <= A.n && !edge ? A.nt / kTc - s : 0;
                     if (kBeam) {
                         beam = A.beam ? A.beam + it.f : nullptr;
                         beam_avg = A.beam_avg;
@@ -432,18 +469,50 @@ xeng_pair_kernel(const __grid_constant__ Params p)
                 item += item_step;
             }
         };
+        // the word at a, without touching bytes outside the array
+        auto load_word = [&](const uint8_t *a) {
+            uint32_t v = 0;
+            if (!edge || (a >= lo && a + 4 <= hi)) {
+                v = __ldg(reinterpret_cast<const uint32_t *>(a));
+            } else {
+                for (int b = 0; b < 4; ++b)
+                    if (a + b >= lo && a + b < hi) v |= uint32_t(__ldg(a + b)) << (8 * b);
+            }
+            return v;
+        };
         uint4 w[kUnits];                       // this thread's samples of the team's next stage
+        uint32_t wx = 0;
         auto load = [&] {
             const uint8_t *a = ptr;
             if (whole > 0) {
 #pragma unroll
-                for (int k = 0; k < kUnits; ++k, a += kRowStep * row_t) w[k] = load16(a);
+                for (int k = 0; k < kUnits; ++k, a += kRowStep * row_t) {
+                    if (kAligned) {
+                        w[k] = load16(a);
+                    } else {
+                        const uint32_t *v = reinterpret_cast<const uint32_t *>(a);
+                        w[k] = make_uint4(__ldg(v), __ldg(v + 1), __ldg(v + 2), __ldg(v + 3));
+                    }
+                }
             } else {
 #pragma unroll
                 for (int k = 0; k < kUnits; ++k, a += kRowStep * row_t) {
                     w[k] = make_uint4(0u, 0u, 0u, 0u);
-                    if (k * kRowStep < rows) w[k] = load16(a);
+                    if (k * kRowStep < rows) {
+                        if (kAligned) {
+                            w[k] = load16(a);
+                        } else {
+                            w[k].x = load_word(a);
+                            if (left + sh > 4) w[k].y = load_word(a + 4);
+                            if (left + sh > 8) w[k].z = load_word(a + 8);
+                            if (left + sh > 12) w[k].w = load_word(a + 12);
+                        }
+                    }
                 }
+            }
+            if (!kAligned) {
+                wx = 0;
+                if (x_rows > 0) wx = load_word(x_ptr);
             }
         };
         enter();
@@ -454,6 +523,8 @@ xeng_pair_kernel(const __grid_constant__ Params p)
         while (more) {
             int32_t *const b_ptr = beam;       // beam of the stage being converted
             const int b_avg = beam_avg, b_ld = beam_ld, b_t = t_beam, b_rows = rows;
+            const int c_left = left, c_shift = 8 * sh;
+            const bool c_skew = skew;
             int pw[kUnits];
             // the next stage of this team
             s += kTeams;
@@ -462,22 +533,47 @@ xeng_pair_kernel(const __grid_constant__ Params p)
                 rows -= rows > 0 ? kTeams * kTc : 0;
                 whole -= kTeams;
                 t_beam += kTeams * kTc;
+                if (!kAligned) {
+                    x_ptr += (long long)(kTeams * kTc) * row_t;
+                    x_rows -= kTeams * kTc;
+                }
             } else {
                 enter();
             }
             more = item < p.n_items;
-            if (!more) rows = whole = 0;
+            if (!more) rows = whole = x_rows = 0;
             if (!mbar_wait(bar_plane_empty(cstage), cphase, abort, p.status, 5, p.wait_limit)) break;
             uint8_t *dst = smem + cstage * kPlaneStageBytes + dst_off;
+            if (!kAligned && c_skew) {
+#pragma unroll
+                for (int k = 0; k < kUnits; ++k) {
+                    const uint32_t next = __shfl_down_sync(0xFFFFFFFFu, w[k].x, 1),
+                                   over = __shfl_sync(0xFFFFFFFFu, wx, 4 * k + (lane >> 3));
+                    w[k].x = __funnelshift_r(w[k].x, w[k].y, c_shift);
+                    w[k].y = __funnelshift_r(w[k].y, w[k].z, c_shift);
+                    w[k].z = __funnelshift_r(w[k].z, w[k].w, c_shift);
+                    w[k].w = __funnelshift_r(w[k].w, c == 7 ? over : next, c_shift);
+                }
+            }
+            if (!kAligned && c_left < 16) {    // bytes past the inputs
+                auto mask = [&](int j) {
+                    const int b = c_left - 4 * j;
+                    return b >= 4 ? 0xFFFFFFFFu : b > 0 ? (1u << (8 * b)) - 1u : 0u;
+                };
+#pragma unroll
+                for (int k = 0; k < kUnits; ++k) {
+                    w[k].x &= mask(0);
+                    w[k].y &= mask(1);
+                    w[k].z &= mask(2);
+                    w[k].w &= mask(3);
+                }
+            }
 #pragma unroll
             for (int k = 0; k < kUnits; ++k) {
                 uint32_t ww[4] = {w[k].x, w[k].y, w[k].z, w[k].w};
                 uint32_t Q[4], R[4], M[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    if (kZeroInvalid) ww[e] = zero_invalid4(ww[e]);
-                    planes4(ww[e], p.one, p.minus_one, p.sixteen, Q[e], R[e], M[e]);
-                }
+                for (int e = 0; e < 4; ++e) planes4<kZeroInvalid>(ww[e], p, Q[e], R[e], M[e]);
                 if (kBeam)
                     pw[k] = power256(ww[0], false, power256(ww[1], false, 0)) +
                             power256(ww[2], false, power256(ww[3], false, 0));
@@ -729,8 +825,10 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool zero_invalid
         std::lock_guard<std::mutex> lock(g_mu);
         if (!g_clusters[dev]) {
             cudaError_t e;
-            for (auto fn : {xeng_pair_kernel<false, false>, xeng_pair_kernel<true, false>,
-                            xeng_pair_kernel<false, true>, xeng_pair_kernel<true, true>}) {
+            for (auto fn : {xeng_pair_kernel<false, false, false>, xeng_pair_kernel<false, true, false>,
+                            xeng_pair_kernel<false, false, true>, xeng_pair_kernel<false, true, true>,
+                            xeng_pair_kernel<true, false, false>, xeng_pair_kernel<true, true, false>,
+                            xeng_pair_kernel<true, false, true>, xeng_pair_kernel<true, true, true>}) {
                 e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBytes);
                 if (e != cudaSuccess) return e;
             }
@@ -742,7 +840,7 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool zero_invalid
     }
     Params prm{};
     long long items = 0;
-    bool beam = false;
+    bool beam = false, aligned = true;
     for (int k = 0; k < count; ++k) {
         const TcArray &A = arrays[k];
         ArrayParams &P = prm.a[k];
@@ -751,6 +849,7 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool zero_invalid
         P.row_t = (long long)P.ld * A.n_chan;
         P.acc = A.acc;
         P.n = A.n;
+        P.n_chan = A.n_chan;
         P.n_blocks = (A.n + 2 * kTile - 1) / (2 * kTile);
         P.nt = A.nt;
         P.n_stages = (A.nt + kTc - 1) / kTc;
@@ -761,6 +860,7 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool zero_invalid
         P.beam_avg = A.beam_avg > 0 ? A.beam_avg : 1;
         P.beam_t0 = A.beam_t0;
         beam = beam || A.beam;
+        aligned = aligned && P.ld % 16 == 0 && (reinterpret_cast<uintptr_t>(A.volt) & 15) == 0;
         items += (long long)A.n_chan * P.n_blocks;
     }
     if (items > 0x3FFFFFFF) return cudaErrorInvalidValue;
@@ -771,12 +871,17 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool zero_invalid
     prm.inject_stall = opt.inject_stall ? 1 : 0;
     prm.one = 1u;
     prm.minus_one = ~0u;
+    prm.fifteen = 15u;
     prm.sixteen = 16u;
     const int grid = 2 * (prm.n_items < g_clusters[dev] ? prm.n_items : g_clusters[dev]);
-    if (zero_invalid)
-        (beam ? xeng_pair_kernel<true, true> : xeng_pair_kernel<true, false>)<<<grid, kThreads, kSmemBytes, s>>>(prm);
-    else
-        (beam ? xeng_pair_kernel<false, true> : xeng_pair_kernel<false, false>)<<<grid, kThreads, kSmemBytes, s>>>(prm);
+    const auto fn = aligned ? (zero_invalid ? (beam ? xeng_pair_kernel<true, true, true> : xeng_pair_kernel<true, true, false>)
+                                            : (beam ? xeng_pair_kernel<true, false, true>
+                                                    : xeng_pair_kernel<true, false, false>))
+                            : (zero_invalid ? (beam ? xeng_pair_kernel<false, true, true>
+                                                    : xeng_pair_kernel<false, true, false>)
+                                            : (beam ? xeng_pair_kernel<false, false, true>
+                                                    : xeng_pair_kernel<false, false, false>));
+    fn<<<grid, kThreads, kSmemBytes, s>>>(prm);
     return cudaGetLastError();
 }
 

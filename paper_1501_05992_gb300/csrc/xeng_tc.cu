@@ -919,6 +919,8 @@ bool tc_supported(int n_inputs, int device)
     return cached[device] == 1;
 }
 
+bool tc_any_rows(int n, TcItems items) { return n > kTile && n <= 2 * kTile && items != TcItems::kSingle; }
+
 cudaError_t launch_group(const TcArray *arrays, int count, bool zero_invalid, int dev,
                          DeviceStatus *status, const TcOptions &opt, cudaStream_t s);
 
@@ -952,8 +954,8 @@ cudaError_t launch_xeng_tc_batch(const TcArray *arrays, int count, DeviceStatus 
         const TcArray &A = arrays[k];
         if (A.nt <= 0) continue;
         const int ld = A.ld ? A.ld : A.n;
-        if (A.nt > kTcMaxSamples || A.n < 1 || ld < A.n || ld % 16 != 0 || A.n_chan < 1 || !A.acc ||
-            (reinterpret_cast<uintptr_t>(A.volt) & 15) != 0)
+        if (A.nt > kTcMaxSamples || A.n < 1 || ld < A.n || A.n_chan < 1 || !A.acc) return cudaErrorInvalidValue;
+        if (!tc_any_rows(A.n, A.items) && (ld % 16 != 0 || (reinterpret_cast<uintptr_t>(A.volt) & 15) != 0))
             return cudaErrorInvalidValue;
     }
     for (int mode = 0; mode < 2; ++mode) {
@@ -1026,7 +1028,7 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool zero_invalid, in
     for (int k = 0; k < count; ++k) {
         const TcArray &A = arrays[k];
         if (A.nt <= 0 || A.zero_invalid != zero_invalid) continue;
-        if (A.n > kTile && A.n <= 2 * kTile && A.items != TcItems::kSingle) {
+        if (tc_any_rows(A.n, A.items)) {
             pair[n_pair++] = A;
         } else {
             order[m++] = k;

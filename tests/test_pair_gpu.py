@@ -58,3 +58,28 @@ def test_pair_extreme_sums_exact(byte):
     # every sample is the same: T times the product of one
     want = oracle.xmac(volt[:1]) * T
     assert np.array_equal(got.cpu().numpy(), oracle.to_int32(want))
+
+
+# rows on every byte offset (odd and even strides, buffers that start off a word
+# boundary, the first and last channels' words over the ends of the buffer), the
+# second tile ending at, before and after a word of its last lane
+@pytest.mark.parametrize("N,F,T", [(131, 1, 70), (159, 4, 129), (201, 3, 64), (250, 6, 333), (251, 2, 65),
+                                   (253, 80, 40), (254, 5, 257), (255, 3, 200)])
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+def test_pair_rows_on_any_byte(N, F, T, offset):
+    if not path_available("tc_fp8", N):
+        pytest.skip("tc_fp8 unsupported")
+    volt = np.random.default_rng(N + F + T + offset).integers(0, 256, (T, F, N), dtype=np.uint8)
+    buf = torch.full((T * F * N + 8,), 0x5A, dtype=torch.uint8, device="cuda")
+    d = buf[offset:offset + T * F * N].view(T, F, N)
+    d.copy_(torch.from_numpy(volt))
+    c = corr.Correlator(N, F, T, path="tc_fp8", zero_invalid=offset == 3)
+    tri, beam = c.integrate_beam(d, 1)
+    c.accumulate(d)
+    acc = c.dump()
+    c.sync()
+    c.close()
+    want = oracle.to_int32(oracle.xmac(volt, offset == 3))
+    assert np.array_equal(tri.cpu().numpy(), want)
+    assert np.array_equal(acc.cpu().numpy(), want)
+    assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, offset == 3))
