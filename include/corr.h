@@ -118,7 +118,8 @@ int corr_set_path(corr_ctx *ctx, int path);
  * and the tile left of it as one 256-row column of the triangle (one
  * conversion of the shared tile feeds two accumulators), and for 129 to 256
  * inputs the whole 256 x 256 block of a channel as one item of a pair of SMs.
- * 0 chooses by shape: 32 when n_inputs <= 32 on the CUDA-core path; on the
+ * 0 chooses by shape: on the CUDA-core path a kernel of 4 x 4 tiles without
+ * staging up to 64 inputs and 65535 channels, else 64; on the
  * tcgen05 path the 256 x 256 block for 129 to 256 inputs, else pair items from
  * 64 stages of 64 samples per launch.  A value that does not apply
  * to the context's path is ignored by it.  Any other value: CORR_E_ARG.  Only

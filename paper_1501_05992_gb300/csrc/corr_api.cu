@@ -244,6 +244,12 @@ int accumulate_to(corr_ctx *c, const uint8_t *volt, int nt, int32_t *target, boo
             if (e != cudaSuccess) return cuda_fail(e);
             fresh = false;
         }
+    } else if (path == CORR_PATH_CUDACORE && c->tile != 32 && c->tile != 64 && c->n <= kSmallMaxInputs &&
+               c->f <= 65535) {
+        prof_begin(c, s);
+        e = launch_xeng_small(volt, c->f, c->n, nt, zi, target, fresh, c->sm_count, s);
+        prof_end(c, CORR_K_XENGINE, s, 1);
+        if (e != cudaSuccess) return cuda_fail(e);
     } else if (path == CORR_PATH_CUDACORE) {
         const StagePlan &P = c->dp4a;
         const size_t plane_max = size_t(P.f_chunk) * (P.t_chunk / 2) * P.n_pad;

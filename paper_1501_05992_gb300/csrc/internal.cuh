@@ -76,6 +76,12 @@ cudaError_t launch_pad_rows(const uint8_t *src, long long rows, int n, int ld, u
 cudaError_t launch_xeng_dp4a(const int32_t *A, const int32_t *W, int n, int n_pad, int fc,
                              int tw_pad, int32_t *acc, int f0, bool fresh, int tile, cudaStream_t s);
 
+// CUDA-core X-engine of n <= kSmallMaxInputs inputs and at most 65535 channels,
+// straight from the packed samples (no staging); stores or adds as above.
+constexpr int kSmallMaxInputs = 64;
+cudaError_t launch_xeng_small(const uint8_t *volt, int n_chan, int n, int nt, bool zero_invalid, int32_t *out,
+                              bool fresh, int sm_count, cudaStream_t s);
+
 // int8 mma.sync X-engine over a staged K-major channel chunk (X and its
 // twisted plane Xt, both [fc][n_pad][t_pad][2]).
 cudaError_t launch_xeng_mma8(const int8_t *X, const int8_t *Xt, int n, int n_pad, int fc,
