@@ -100,29 +100,23 @@ int corr_destroy(corr_ctx *ctx);
 
 /* Select the implementation.  CORR_E_UNSUPPORTED if the path cannot run on
  * this device (CORR_PATH_TC_FP8 needs an sm_103 device).  The tensor-core
- * path reads the rows of 129 to 256 inputs (tile 0 or 256, corr_set_tile) as
- * they are, on any byte boundary; other rows come through TMA, which needs
- * them on 16-byte boundaries: with n_inputs % 16 != 0 each call's samples are
- * first copied into rows of round_up(n_inputs, 16) bytes in the workspace (up
- * to 4 GiB: a whole integration where it fits, else chunks of a multiple of 64
- * samples).  In a batch, arrays with n_inputs % 16 != 0 are correlated in
- * launches of their own.  AUTO picks the tensor-core path from
- * 64 inputs on.  Valid only between integrations (corr_samples() == 0), else
- * CORR_E_STATE.  The default is CORR_PATH_AUTO. */
+ * path reads the rows of up to 256 inputs as they are, on any byte boundary;
+ * longer rows come through TMA, which needs them on 16-byte boundaries: with
+ * n_inputs % 16 != 0 each call's samples are first copied into rows of
+ * round_up(n_inputs, 16) bytes in the workspace (up to 4 GiB: a whole
+ * integration where it fits, else chunks of a multiple of 64 samples).  In a
+ * batch, arrays with n_inputs % 16 != 0 are correlated in launches of their
+ * own.  AUTO picks the tensor-core path from 64 inputs on.  Valid only between
+ * integrations (corr_samples() == 0), else CORR_E_STATE.  The default is
+ * CORR_PATH_AUTO. */
 int corr_set_path(corr_ctx *ctx, int path);
 
 /* Tile shape (Section 3.4.2, Eq. 4: the tile sets the arithmetic intensity).
- * CUDA-core path: 32 or 64 inputs per side.  tcgen05 path: 128 = every work
- * item one 128 x 128 tile pair (one TMEM accumulator each, so an item's
- * epilogue overlaps the next item's MMAs); 256 = pair items, a diagonal tile
- * and the tile left of it as one 256-row column of the triangle (one
- * conversion of the shared tile feeds two accumulators), and for 129 to 256
- * inputs the whole 256 x 256 block of a channel as one item of a pair of SMs.
- * 0 chooses by shape: on the CUDA-core path a kernel of 4 x 4 tiles without
- * staging up to 64 inputs and 65535 channels, else 64; on the
- * tcgen05 path the 256 x 256 block for 129 to 256 inputs, else pair items from
- * 64 stages of 64 samples per launch.  A value that does not apply
- * to the context's path is ignored by it.  Any other value: CORR_E_ARG.  Only
+ * CUDA-core path: 32 or 64 inputs per side, or 0 to choose by shape: a kernel
+ * of 4 x 4 tiles without operand staging up to 64 inputs and 65535 channels,
+ * else 64.  128 and 256 are accepted for the tcgen05 path, which chooses its
+ * work items itself (256-input blocks on the diagonal, the tiles off them, a
+ * last tile alone); no value changes it.  Any other value: CORR_E_ARG.  Only
  * between integrations (CORR_E_STATE). */
 int corr_set_tile(corr_ctx *ctx, int tile);
 
@@ -271,8 +265,9 @@ int corr_unpack(const uint8_t *d_volt, int n_time, int n_chan, int n_inputs,
  * Several arrays of uneven size correlated together (the MWA correlator runs
  * one X-engine per GPU over a fixed set of channels, Section 3.4; here one
  * GPU serves several arrays).  Arrays on the tensor-core path are correlated
- * by ONE persistent launch (up to CORR_BATCH_TC_GROUP arrays per launch; the
- * work items of all of them, longest first, shared by every SM); arrays on
+ * together, up to CORR_BATCH_TC_GROUP of them per persistent launch (one launch
+ * per kind of work item: 256-input blocks, the tiles off them, a last tile
+ * alone; the items of all arrays, longest first, shared by every SM); arrays on
  * other paths get their own kernels on the same stream.
  */
 #define CORR_BATCH_MAX 16
@@ -322,7 +317,7 @@ int corr_batch_dump(corr_batch *b, int32_t *const *d_vis, void *stream);
 
 /*
  * corr_integrate for every array a with d_vis[a] != NULL, the tensor-core
- * arrays sharing one persistent launch: array a's n_time[a] samples of
+ * arrays sharing persistent launches: array a's n_time[a] samples of
  * d_volt[a] become the triangle in d_vis[a].  Running integrations are not
  * touched.  All checks happen before anything is enqueued.
  */

@@ -38,7 +38,7 @@ struct corr_ctx {
     int n = 0, f = 0, t_max = 0;
     int device = 0, sm_major = 0, sm_minor = 0, sm_count = 0;
     int path = CORR_PATH_AUTO;
-    int tile = 0;            // CUDA-core tile (32 or 64) or tcgen05 items (128, 256); 0 = chosen by shape
+    int tile = 0;            // CUDA-core tile (32 or 64); 0 = chosen by shape; 128, 256: no effect
     long long wait_limit = 0;   // device bounded-wait limit (cycles), 0 = default
     bool inject_stall = false;  // one-shot test hook for the next tensor-core launch
     unsigned flags = 0;
@@ -180,12 +180,6 @@ void prof_end(corr_ctx *c, int kind, cudaStream_t s, int launches)
     c->prof_cur = {nullptr, nullptr};
 }
 
-// Work-item shape of the tensor-core path chosen by corr_set_tile.
-TcItems tc_items(const corr_ctx *c)
-{
-    return c->tile == 128 ? TcItems::kSingle : c->tile == 256 ? TcItems::kPairs : TcItems::kAuto;
-}
-
 // Order `s` after a host dump that may still be reading the accumulators.
 int wait_host_dump(corr_ctx *c, cudaStream_t s)
 {
@@ -216,7 +210,7 @@ int accumulate_to(corr_ctx *c, const uint8_t *volt, int nt, int32_t *target, boo
         // rows of n % 16 != 0 inputs go through a padded copy, chunk by chunk, except
         // where the kernel reads them as they are
         if (c->n % 16 == 0 && (reinterpret_cast<uintptr_t>(volt) & 15) != 0) return CORR_E_ARG;
-        const int pad_t = tc_any_rows(c->n, tc_items(c)) ? 0 : tc_pad_samples(c->n, c->f, c->t_max);
+        const int pad_t = tc_any_rows(c->n) ? 0 : tc_pad_samples(c->n, c->f, c->t_max);
         const int step = pad_t ? (pad_t < kTcMaxSamples ? pad_t : kTcMaxSamples) : kTcMaxSamples;
         for (int t0 = 0; t0 < nt; t0 += step) {
             const int ntc = nt - t0 < step ? nt - t0 : step;
@@ -235,12 +229,13 @@ int accumulate_to(corr_ctx *c, const uint8_t *volt, int nt, int32_t *target, boo
             opt.wait_limit = c->wait_limit;
             opt.inject_stall = c->inject_stall;
             c->inject_stall = false;
-            TcArray arr{src, target, c->f, c->n, ntc, zi, fresh, tc_items(c), ld};
+            TcArray arr{src, target, c->f, c->n, ntc, zi, fresh, ld};
             arr.beam = beam;
             arr.beam_avg = beam_avg;
             arr.beam_t0 = t0;
-            e = launch_xeng_tc_batch(&arr, 1, c->status, opt, s);
-            prof_end(c, CORR_K_XENGINE, s, 1);
+            int launches = 0;
+            e = launch_xeng_tc_batch(&arr, 1, c->status, opt, s, &launches);
+            prof_end(c, CORR_K_XENGINE, s, launches);
             if (e != cudaSuccess) return cuda_fail(e);
             fresh = false;
         }
@@ -999,7 +994,6 @@ int batch_correlate(corr_batch *b, const uint8_t *const *d_volt, const int *n_ti
                 arr[k].nt = ntc;
                 arr[k].zero_invalid = (c->flags & CORR_ZERO_INVALID) != 0;
                 arr[k].fresh = t0 == 0 ? (into ? true : c->fresh) : false;
-                arr[k].items = tc_items(c);
                 ++k;
             }
             TcOptions opt;
@@ -1007,8 +1001,9 @@ int batch_correlate(corr_batch *b, const uint8_t *const *d_volt, const int *n_ti
             opt.inject_stall = lead->inject_stall;
             lead->inject_stall = false;
             prof_begin(lead, s);
-            cudaError_t e = launch_xeng_tc_batch(arr, k, lead->status, opt, s);
-            prof_end(lead, CORR_K_XENGINE, s, 1);
+            int launches = 0;
+            cudaError_t e = launch_xeng_tc_batch(arr, k, lead->status, opt, s, &launches);
+            prof_end(lead, CORR_K_XENGINE, s, launches);
             if (e != cudaSuccess) return cuda_fail(e);
         }
         if (!into) {

@@ -93,33 +93,29 @@ struct TcOptions {
     long long wait_limit = 0;   // bounded-wait limit in clock64 cycles (0: about 1 s)
     bool inject_stall = false;  // test hook: make the launch's first wait expire
 };
-// Work items of the tensor-core path: single 128 x 128 tile pairs, pair items
-// (a diagonal tile and the tile left of it, sharing one conversion), or
-// pairs only on launches of at least 64 stages.
-enum class TcItems { kAuto = 0, kSingle = 1, kPairs = 2 };
 struct TcArray {
     const uint8_t *volt;   // [nt][n_chan][ld] packed voltages (n used of each row of ld bytes)
     int32_t *acc;          // [n_chan][P][2] accumulators
     int n_chan, n, nt;
     bool zero_invalid, fresh;
-    TcItems items = TcItems::kAuto;
-    int ld = 0;            // row stride in bytes (0: n); a multiple of 16 unless tc_any_rows()
+    int ld = 0;            // row stride in bytes (0: n); a multiple of 16 unless tc_any_rows(n)
     // incoherent beam of the same samples, added into beam[(beam_t0 + t) /
     // beam_avg][n_chan] (zeroed by the caller); NULL for none
     int32_t *beam = nullptr;
     int beam_avg = 1, beam_t0 = 0;
 };
-// Whether an array of n inputs runs on the CTA-pair kernel (xeng_pair.cu), which
-// takes rows on any byte boundary.
-bool tc_any_rows(int n, TcItems items);
+// Whether the tensor-core path takes an array of n inputs with its rows on any byte
+// boundary (up to 256 inputs; the others come through TMA).
+bool tc_any_rows(int n);
 // Samples per padded copy for the tensor-core path when n % 16 != 0: the
 // whole integration if it fits kTcPadCap bytes, else chunks of a multiple
 // of 64 samples.
 constexpr size_t kTcPadCap = size_t(4) << 30;
-// One persistent launch over every (channel, tile pair) of up to
-// kTcMaxArrays arrays (nt <= kTcMaxSamples each; arrays with nt == 0 skipped).
+// Persistent launches over every channel and tile of up to kTcMaxArrays arrays (nt <=
+// kTcMaxSamples each; arrays with nt == 0 skipped).  *launches receives the number of
+// kernels enqueued.
 cudaError_t launch_xeng_tc_batch(const TcArray *arrays, int count, DeviceStatus *status,
-                                 const TcOptions &opt, cudaStream_t s);
+                                 const TcOptions &opt, cudaStream_t s, int *launches);
 
 // Incoherent beam: out[k][f] = sum of |x|^2 over inputs and the n_avg samples
 // of block k (n_time / n_avg blocks), int32.

@@ -83,3 +83,37 @@ def test_pair_rows_on_any_byte(N, F, T, offset):
     assert np.array_equal(tri.cpu().numpy(), want)
     assert np.array_equal(acc.cpu().numpy(), want)
     assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, offset == 3))
+
+
+# tiles off the 256-input blocks and a last tile alone: one input past a block, an
+# odd number of tiles, a ragged last tile in and off a block; the input counts that
+# are no multiple of 16 run on padded rows; T around a stage and the teams' turns
+@pytest.mark.parametrize("N,F,T", [(257, 2, 63), (272, 1, 65), (384, 3, 128), (400, 2, 129), (512, 80, 100),
+                                   (513, 1, 200), (640, 2, 64), (700, 1, 1), (1024, 1, 321)])
+def test_tiles_off_the_blocks_exact(N, F, T):
+    _check_all_calls(N, F, T, zero_invalid=N % 3 == 0)
+
+
+# a single tile: its inputs' last 16 columns, rows on any byte, channels past the SMs
+@pytest.mark.parametrize("N,F,T", [(1, 2, 70), (15, 3, 65), (16, 1, 64), (49, 2, 300), (64, 160, 129), (97, 1, 63),
+                                   (113, 2, 257), (127, 5, 130), (128, 310, 65)])
+def test_single_tiles_exact(N, F, T):
+    _check_all_calls(N, F, T, zero_invalid=N % 2 == 0)
+
+
+def _check_all_calls(N, F, T, zero_invalid):
+    if not path_available("tc_fp8", N):
+        pytest.skip("tc_fp8 unsupported")
+    volt = np.random.default_rng(N + F + T).integers(0, 256, (T, F, N), dtype=np.uint8)
+    c = corr.Correlator(N, F, 2 * T, path="tc_fp8", zero_invalid=zero_invalid)
+    d = torch.from_numpy(volt).cuda()
+    tri, beam = c.integrate_beam(d, 1)
+    c.accumulate(d)
+    c.accumulate(d)
+    acc = c.dump()
+    c.sync()
+    c.close()
+    vis = oracle.xmac(volt, zero_invalid)
+    assert np.array_equal(tri.cpu().numpy(), oracle.to_int32(vis))
+    assert np.array_equal(acc.cpu().numpy(), oracle.to_int32(2 * vis))
+    assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
