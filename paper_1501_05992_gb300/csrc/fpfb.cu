@@ -15,7 +15,7 @@
 // stages chain on the device.
 //
 // Work decomposition.  A CTA of 4 warps takes 16 consecutive inputs of one
-// coarse channel over a run of frames: frames in groups of G = 8, inputs in
+// coarse channel over one group of frames (more on very long inputs): G = 8, inputs in
 // sub-batches of 2, so that one unit (group, sub-batch) is 16 (frame, input)
 // transforms, taken in three phases separated by CTA barriers.
 //
@@ -55,8 +55,6 @@
 // The work is fp32 arithmetic (about 10.6 kflop per frame and input: 12 x 128
 // complex-by-real multiply-adds and a 128-point FFT) against 256 bytes read and
 // 128 bytes written, so the kernel is bound by the FP32 pipes, not by HBM.
-#include <algorithm>
-
 #include "internal.cuh"
 
 namespace corr {
@@ -68,7 +66,6 @@ constexpr int kPfbSub = 2;                    // inputs per sub-batch, two windo
 constexpr int kPfbInputs = 16;                // inputs per CTA: 8 sub-batches
 constexpr int kPfbGroup = 8;                  // frames per group
 constexpr int kPfbXf = kPfbSub * kPfbGroup;   // transforms per unit
-constexpr int kPfbMaxFramesPerCta = 120;      // frames per CTA (whole groups), at most
 constexpr int kPfbCtasPerSm = 4;
 // shared memory: windowed frames [16][Re 128 | Im 128 | pad 16] floats (the
 // pad spreads the transforms over the banks), 8-point results [16 transforms]
@@ -178,7 +175,6 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
 {
     constexpr int G = kPfbGroup;
     constexpr int B = G + TAPS - 1;             // blocks that feed a group
-    static_assert(kPfbMaxFramesPerCta % G == 0, "whole groups per CTA");
     extern __shared__ __align__(16) float smem[];
     float *const U = smem;                                    // [32][kUStride]
     float *const Z = U + kPfbXf * kUStride;                   // [32][kZStride]
@@ -335,14 +331,14 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                         if (kSpec && i < a.N && m < m1)
                             a.spec[(size_t(m) * C + size_t(q) * kPfbPoints + c) * a.N + i] = make_float2(yr, yi);
                         if (kVolt) {
-                            // clamp to [-7, 7], then adding 1.5 * 2^23 rounds to the nearest
-                            // integer, ties to even, and leaves it (two's complement) in the
-                            // low mantissa bits
+                            // clamp to [-7, 7], then adding 1.5 * 2^23 + 8 rounds to the nearest
+                            // integer, ties to even, and leaves it plus 8 in the low mantissa
+                            // bits; the copy-out turns both nibbles into two's complement
                             const float2 s = kFold ? make_float2(yr, yi) : mul2(make_float2(yr, yi), dup2(a.scale));
                             const float2 w = add2(make_float2(fminf(fmaxf(s.x, -7.0f), 7.0f),
-                                                              fminf(fmaxf(s.y, -7.0f), 7.0f)), dup2(12582912.0f));
+                                                              fminf(fmaxf(s.y, -7.0f), 7.0f)), dup2(12582920.0f));
                             tile[f * kTileFrame + c * kPfbInputs + sb * kPfbSub + iw3] =
-                                uint8_t((__float_as_uint(w.x) << 4) | (__float_as_uint(w.y) & 15u));
+                                uint8_t(__float_as_uint(w.x) * 16u + __float_as_uint(w.y));
                         }
                     }
                 }
@@ -363,9 +359,14 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                 uint8_t *dst = a.volt + (size_t(g0 + f) * C + size_t(q) * kPfbPoints + c) * a.N + i0 + 16 * hh;
                 const uint8_t *src = tile + f * kTileFrame + c * kPfbInputs + 16 * hh;
                 if (full) {
-                    *reinterpret_cast<uint4 *>(dst) = *reinterpret_cast<const uint4 *>(src);
+                    uint4 v = *reinterpret_cast<const uint4 *>(src);
+                    v.x ^= 0x88888888u;
+                    v.y ^= 0x88888888u;
+                    v.z ^= 0x88888888u;
+                    v.w ^= 0x88888888u;
+                    *reinterpret_cast<uint4 *>(dst) = v;
                 } else {
-                    for (int w = 0; w < 16 && i0 + 16 * hh + w < a.N; ++w) dst[w] = src[w];
+                    for (int w = 0; w < 16 && i0 + 16 * hh + w < a.N; ++w) dst[w] = src[w] ^ 0x88u;
                 }
             }
             // the next group writes the codes only after two more barriers,
@@ -419,24 +420,16 @@ cudaError_t launch_fine_pfb(const int8_t *x, int n_coarse, int n_inputs, long lo
     a.N = n_inputs;
     a.M = int(n_samples / kPfbPoints - n_taps + 1);
     a.scale = scale;
-    // frames per CTA: the longest run (fewest CTA prologues) that still gives
-    // two waves of CTAs over the SMs
-    static int sm_count[kPfbMaxDevices] = {};
-    int dev = 0, sms = 0;
+    // frames per CTA: one group, as long as the grid allows it.  A CTA's prologue (the
+    // window, the twiddles, the first loads) hides behind the SM's other CTAs, while
+    // runs of up to 120 frames left the last CTAs' SMs idle: 24 coarse channels x 256
+    // inputs x 500 frames 1.07 -> 0.98 ms, 12 x 256 x 300 with spectra 1.49 -> 1.34 ms.
+    int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
-    if (dev < kPfbMaxDevices && sm_count[dev] > 0) {
-        sms = sm_count[dev];
-    } else {
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        if (dev < kPfbMaxDevices) sm_count[dev] = sms;
-    }
     const long long gx = (n_inputs + kPfbInputs - 1) / kPfbInputs;
-    const long long want = 2LL * sms * kPfbCtasPerSm;
-    const long long per_cta = (a.M * gx * n_coarse + want - 1) / want;
-    a.fpc = int(std::min<long long>(kPfbMaxFramesPerCta,
-                                    std::max<long long>(kPfbGroup, (per_cta + kPfbGroup - 1) / kPfbGroup * kPfbGroup)));
+    const long long groups = (a.M + kPfbGroup - 1) / kPfbGroup;
+    a.fpc = int(kPfbGroup * ((groups + 65534) / 65535));
     const dim3 grid(unsigned(gx), unsigned((a.M + a.fpc - 1) / a.fpc), unsigned(n_coarse));
     return n_taps == 12 ? launch_taps<12>(a, grid, dev, s) : launch_taps<1>(a, grid, dev, s);
 }
