@@ -379,21 +379,6 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t tmem, uint32_t cols)
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols));
 }
 
-// 256 (r^2 + m^2) summed over the 4 packed samples of w, plus acc: the high
-// nibble with the low one cleared is the signed byte 16 r, the low nibble
-// moved up the signed byte 16 m (Appendix A: two's complement, real high).
-// With zero_invalid, samples with a nibble of 8 count as zero.
-__device__ __forceinline__ int power256(uint32_t w, bool zero_invalid, int acc)
-{
-    uint32_t hr = w & 0xF0F0F0F0u, hm = (w << 4) & 0xF0F0F0F0u;
-    if (zero_invalid) {
-        const uint32_t bad = __vcmpeq4(hr, 0x80808080u) | __vcmpeq4(hm, 0x80808080u);
-        hr &= ~bad;
-        hm &= ~bad;
-    }
-    return __dp4a(int(hm), int(hm), __dp4a(int(hr), int(hr), acc));
-}
-
 }  // namespace
 
 // One launch over every channel of up to kTcMaxArrays arrays, storing (fresh) or
