@@ -44,7 +44,7 @@
 // integration: MMAs (two thirds of that kernel's) and instructions.  The
 // shared-memory pipe is 70 % busy, the tensor pipe 63 %, the ALU pipe 50 %.  Short
 // launches are bound by the epilogue's exchange and stores (adding 500 samples to the
-// full band's triangle: 0.41 ms, 0.28 ms of it what the adds take in L2).  One tile
+// full band's triangle: 0.38 ms, of which 0.28 ms is what the adds alone take in L2).  One tile
 // alone is bound by its MMAs (M=128 N=128 reads 8 KB of operands in 64 cycles) and
 // loads: 128 inputs x 1520 channels x 5000 samples 0.33 -> 0.31 ms, 500 samples added
 // to 768 channels 67 -> 35 us.
@@ -76,8 +76,15 @@
 // distributed shared memory into CTA 0's inbox, CTA 1 the others, whose W[j][i]
 // CTA 0 sends (st.async, counted by the inbox's barrier: plain stores and a
 // cluster-scope release wait for the thread's stores to the output too, 0.36
-// against 0.33 ms for 500 samples of the full band).  TMEM holds two 256-column
-// accumulators, so an item's epilogue overlaps the next item's main loop.
+// against 0.33 ms for 500 samples of the full band).  Of that half both operands
+// are in shared memory, so that any warp can emit any of it: the quarters' shares of the
+// diagonal tile are as 4 : 3 : 2 : 1 (j <= i), and its pieces go to the warps that
+// have less, while TMEM is already free (500 samples of the full band 0.323 ->
+// 0.295 ms, added 0.408 -> 0.383 ms, against halves emitted by quarter after a wait of
+// all warps; one 1.28 MHz channel of 5000 samples 74.4 -> 72.6 us; 250 inputs lose
+// 0.8 % on long integrations, which no arrangement of the
+// same loops that was tried avoids for both kinds of rows).  TMEM holds two
+// 256-column accumulators, so an item's epilogue overlaps the next item's main loop.
 #pragma once
 
 #include <mutex>
@@ -113,17 +120,22 @@ constexpr long long kDefaultWaitLimit = 1LL << 31;
 
 // shared-memory map (offsets from the 1024-aligned base, the same in both CTAs)
 constexpr int kSmPlanes = 0;
-constexpr int kSmXch = kSmPlanes + kPlaneStages * kPlaneStageBytes;
-// exchange buffers: the CTA's own (128 rows of 128 floats) and its inbox (64
-// rows), padded by 16 bytes a row so that 16-byte stores down the rows spread
-// over the banks
-constexpr int kXchPitch = kTile * 4 + 16, kInboxRows = 64;
-constexpr int kSmInbox = kSmXch + kTile * kXchPitch;
-constexpr int kSmBars = kSmInbox + kInboxRows * kXchPitch;
+// epilogue buffers: the CTA's diagonal tile (W[i][j]: row i holds the columns up to the
+// end of its quarter, 32 q + 32), its own operand of its half of the off-diagonal tile
+// (64 rows i of 128 columns j), and its inbox for the pair's operand; rows are padded
+// by 16 bytes so that 16-byte stores down the rows spread over the banks
+constexpr int kSmDiag = kSmPlanes + kPlaneStages * kPlaneStageBytes;
+constexpr int kHalfPitch = kTile * 4 + 16, kHalfRows = 64;
+constexpr int kDiagBytes = 32 * (4 * 16 + (32 + 64 + 96 + 128) * 4);
+__device__ __forceinline__ int diag_pitch(int quarter) { return 128 * quarter + 144; }
+__device__ __forceinline__ int diag_base(int quarter) { return 32 * (144 * quarter + 64 * quarter * (quarter - 1)); }
+constexpr int kSmOwn = kSmDiag + kDiagBytes;
+constexpr int kSmInbox = kSmOwn + kHalfRows * kHalfPitch;
+constexpr int kSmBars = kSmInbox + kHalfRows * kHalfPitch;
 constexpr int kNumBars = 2 * kPlaneStages + 4 + 4;
 constexpr int kSmMisc = kSmBars + kNumBars * 8;
 constexpr int kSmemBytes = kSmMisc + 128;
-constexpr int kInboxBytes = kInboxRows * kTile * 4;                // sent per item
+constexpr int kInboxBytes = kHalfRows * kTile * 4;                // sent per item
 static_assert(kSmemBytes <= 227 * 1024, "shared memory");
 
 struct ArrayParams {
@@ -236,7 +248,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
         mbar_init(bar_drain, 1);
         mbar_init(bar_never, 1);
         mbar_init(bar_in_full, 1);
-        mbar_init(bar_in_free, kEpiWarps * 32);
+        mbar_init(bar_in_free, kEpiWarps);
         *abort = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
@@ -564,127 +576,139 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
             fence_after();
             const uint32_t taddr = tmem + uint32_t(slot * kSlotCols) + (uint32_t(q * 32) << 16);
 
-            // W[i][j] (times 2^-18) of this lane's row i into row `row` of this CTA's
-            // buffer, columns j < cols; the quarter's two warps take 32 columns in turn
-            auto put_row = [&](int row, uint32_t tcol, int cols) {
-#pragma unroll 1
-                for (int c0 = 32 * wp; c0 < cols; c0 += 64) {
+            // operands into shared memory, 32 columns of the accumulator at a time: this
+            // lane's row into `row`, or (transposed) its column of the rows there
+            auto put_row = [&](uint8_t *row, uint32_t tcol) {
 #pragma unroll
-                    for (int h = 0; h < 32; h += 16) {
-                        uint32_t v[16];
-                        tmem_ld16(taddr + tcol + c0 + h, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int k = 0; k < 16; k += 4)
-                            *reinterpret_cast<uint4 *>(smem + kSmXch + row * kXchPitch + (c0 + h + k) * 4) =
-                                make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
-                    }
-                }
-            };
-            // outputs (i, j), i = i0 + row for rows [r0, r1) in steps of 16 shared by the
-            // quarter's two warps, j = j0 + il: W[i][j] from row `row - y0` of the buffer
-            // at y, W[j][i] from TMEM column tcol + row (or, x_smem, from the inbox's row
-            // `row - y0`); diag: only j <= i
-            auto emit = [&](int i0, int j0, int r0, int r1, int y0, const uint8_t *y, uint32_t tcol, bool x_smem,
-                            bool diag) {
-#pragma unroll 1
-                for (int c0 = r0 + 16 * wp; c0 < r1 && i0 + c0 < n_in; c0 += 32) {
-                    uint32_t xr[16];
-                    float yv[16];
-                    const uint8_t *yp = y + (c0 - y0) * kXchPitch + il * 4;
-                    if (x_smem) {
-                        const uint8_t *xp = smem + kSmInbox + (c0 - y0) * kXchPitch + il * 4;
-#pragma unroll
-                        for (int k = 0; k < 16; ++k) xr[k] = *reinterpret_cast<const uint32_t *>(xp + k * kXchPitch);
-                    } else {
-                        tmem_ld16(taddr + tcol + c0, xr);
-                    }
-#pragma unroll
-                    for (int k = 0; k < 16; ++k) yv[k] = *reinterpret_cast<const float *>(yp + k * kXchPitch);
-                    if (!x_smem) tmem_wait_ld();
-                    int2 v[16];
-#pragma unroll
-                    for (int k = 0; k < 16; k += 2) {
-                        // exact: the sum and difference are 2 Re and 2 Im times 2^-18, integers
-                        // of at most 256 T <= 2^23 before the scale; adding 1.5 * 2^23 to Re, Im
-                        // leaves them in the encoding's low bits
-                        const float2 x = make_float2(__uint_as_float(xr[k]), __uint_as_float(xr[k + 1]));
-                        const float2 yy = make_float2(yv[k], yv[k + 1]);
-                        const float2 big = make_float2(12582912.0f, 12582912.0f);
-                        const float2 half = make_float2(131072.0f, 131072.0f);
-                        const float2 re = __ffma2_rn(__fadd2_rn(x, yy), half, big);
-                        const float2 im = __ffma2_rn(__ffma2_rn(yy, make_float2(-1.0f, -1.0f), x), half, big);
-                        v[k] = make_int2(__float_as_int(re.x) - 0x4B400000, __float_as_int(im.x) - 0x4B400000);
-                        v[k + 1] = make_int2(__float_as_int(re.y) - 0x4B400000, __float_as_int(im.y) - 0x4B400000);
-                    }
-                    const int ic = i0 + c0;
-                    put_rows16<kFresh>(out_f, ic, j0 + il, n_in, lane,
-                                       ic + 15 < n_in && (!diag || c0 >= 32 * q + 32), v);
-                }
-            };
-
-            // the other operand of the pair's half of the off-diagonal tile, into its
-            // inbox; this CTA's inbox is armed for as many bytes
-            if (kPair && warp == 0 && lane == 0) mbar_expect_tx(bar_in_full, kInboxBytes);
-            if (!kPair) {
-            } else if (rank == 1) {
-                if (q < 2) {                               // W[i][j], rows i < 64 of tile 1
-#pragma unroll 1
-                    for (int c0 = 16 * wp; c0 < kTile; c0 += 32) {
-                        uint32_t v[16];
-                        tmem_ld16(taddr + c0, v);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int k = 0; k < 16; k += 4)
-                            store_async4(peer_inbox + uint32_t(il * kXchPitch + (c0 + k) * 4), v + k, peer_full);
-                    }
-                }
-            } else {                                       // W[j][i], rows i >= 64, transposed
-#pragma unroll 1
-                for (int c0 = 16 * wp; c0 < 64; c0 += 32) {
+                for (int h = 0; h < 32; h += 16) {
                     uint32_t v[16];
-                    tmem_ld16(taddr + kTile + 64 + c0, v);
+                    tmem_ld16(taddr + tcol + h, v);
                     tmem_wait_ld();
 #pragma unroll
-                    for (int k = 0; k < 16; ++k)
-                        store_async(peer_inbox + uint32_t((c0 + k) * kXchPitch + il * 4), v[k], peer_full);
+                    for (int k = 0; k < 16; k += 4)
+                        *reinterpret_cast<uint4 *>(row + (h + k) * 4) = make_uint4(v[k], v[k + 1], v[k + 2], v[k + 3]);
+                }
+            };
+            // outputs (ic + k, j), k < 16, from x[k] = W[j][ic + k] and y[k] = W[ic + k][j]
+            auto emit16 = [&](int ic, int j, const uint32_t (&xr)[16], const float (&yv)[16], bool full) {
+                int2 v[16];
+#pragma unroll
+                for (int k = 0; k < 16; k += 2) {
+                    // exact: the sum and difference are 2 Re and 2 Im times 2^-18, integers
+                    // of at most 256 T <= 2^23 before the scale; adding 1.5 * 2^23 to Re, Im
+                    // leaves them in the encoding's low bits
+                    const float2 x = make_float2(__uint_as_float(xr[k]), __uint_as_float(xr[k + 1]));
+                    const float2 yy = make_float2(yv[k], yv[k + 1]);
+                    const float2 big = make_float2(12582912.0f, 12582912.0f);
+                    const float2 half = make_float2(131072.0f, 131072.0f);
+                    const float2 re = __ffma2_rn(__fadd2_rn(x, yy), half, big);
+                    const float2 im = __ffma2_rn(__ffma2_rn(yy, make_float2(-1.0f, -1.0f), x), half, big);
+                    v[k] = make_int2(__float_as_int(re.x) - 0x4B400000, __float_as_int(im.x) - 0x4B400000);
+                    v[k + 1] = make_int2(__float_as_int(re.y) - 0x4B400000, __float_as_int(im.y) - 0x4B400000);
+                }
+                put_rows16<kFresh>(out_f, ic, j, n_in, lane, full, v);
+            };
+
+            if (kPair) {
+                // the pair's operand of its half of the off-diagonal tile, into its inbox
+                // (this CTA's inbox is armed for as many bytes), and the own operand
+                if (warp == 0 && lane == 0) mbar_expect_tx(bar_in_full, kInboxBytes);
+                if (rank == 1) {
+                    if (q < 2) {                           // W[i][j], rows i < 64 of tile 1
+#pragma unroll 1
+                        for (int c0 = 16 * wp; c0 < kTile; c0 += 32) {
+                            uint32_t v[16];
+                            tmem_ld16(taddr + c0, v);
+                            tmem_wait_ld();
+#pragma unroll
+                            for (int k = 0; k < 16; k += 4)
+                                store_async4(peer_inbox + uint32_t(il * kHalfPitch + (c0 + k) * 4), v + k, peer_full);
+                        }
+                    } else {                               // W[i][j], rows i >= 64
+#pragma unroll 1
+                        for (int c0 = 32 * wp; c0 < kTile; c0 += 64)
+                            put_row(smem + kSmOwn + (il - 64) * kHalfPitch + c0 * 4, c0);
+                    }
+                } else {                                   // W[j][i], transposed
+#pragma unroll 1
+                    for (int c0 = 16 * wp; c0 < 64; c0 += 32) {
+                        uint32_t v[16];
+                        tmem_ld16(taddr + kTile + 64 + c0, v);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            store_async(peer_inbox + uint32_t((c0 + k) * kHalfPitch + il * 4), v[k], peer_full);
+                    }
+#pragma unroll 1
+                    for (int c0 = 16 * wp; c0 < 64; c0 += 32) {
+                        uint32_t v[16];
+                        tmem_ld16(taddr + kTile + c0, v);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int k = 0; k < 16; ++k)
+                            *reinterpret_cast<uint32_t *>(smem + kSmOwn + (c0 + k) * kHalfPitch + il * 4) = v[k];
+                    }
                 }
             }
             // the CTA's own diagonal tile
             const int t0 = it.base + rank * kTile;
-            put_row(il, uint32_t(rank * kTile), 32 * q + 32);
+            const uint32_t tdiag = uint32_t(rank * kTile);
+#pragma unroll 1
+            for (int c0 = 32 * wp; c0 < 32 * q + 32; c0 += 64)
+                put_row(smem + kSmDiag + diag_base(q) + lane * diag_pitch(q) + c0 * 4, tdiag + c0);
             named_sync(2, kEpiWarps * 32);
-            emit(t0, t0, 32 * q, kTile, 0, smem + kSmXch, uint32_t(rank * kTile), false, true);
-            // this CTA's half of the off-diagonal tile
-            auto release_tmem = [&] {          // this accumulator can take the next item but one
-                fence_before();
-                __syncwarp();
-                if (lane == 0) {
-                    if (kPair) remote_arrive(map_rank(bar_acc_empty(slot), 0));
-                    else mbar_arrive(bar_acc_empty(slot));
+            // columns j = il, rows from the start of the quarter on, 16 at a time
+#pragma unroll 1
+            for (int c0 = 32 * q + 16 * wp; c0 < kTile && t0 + c0 < n_in; c0 += 32) {
+                uint32_t xr[16];
+                float yv[16];
+                const int rq = c0 >> 5, pitch = diag_pitch(rq);
+                const uint8_t *yp = smem + kSmDiag + diag_base(rq) + (c0 & 31) * pitch + il * 4;
+                tmem_ld16(taddr + tdiag + c0, xr);
+#pragma unroll
+                for (int k = 0; k < 16; ++k) yv[k] = *reinterpret_cast<const float *>(yp + k * pitch);
+                tmem_wait_ld();
+                emit16(t0 + c0, t0 + il, xr, yv, t0 + c0 + 15 < n_in && c0 >= 32 * q + 32);
+            }
+            // this accumulator can take the next item but one
+            fence_before();
+            __syncwarp();
+            if (lane == 0) {
+                if (kPair) remote_arrive(map_rank(bar_acc_empty(slot), 0));
+                else mbar_arrive(bar_acc_empty(slot));
+            }
+            if (kPair) {
+                // this CTA's half of the off-diagonal tile, both operands in shared memory:
+                // 16 pieces of 16 rows and 32 columns, the more to a warp the fewer its
+                // quarter has of the diagonal tile (4, 3, 2, 1)
+                const int e0 = wp ? 6 + q * (q + 1) / 2 : q * (q - 1) / 2, e1 = e0 + q + wp;
+                if (e0 < e1) {
+                    ok = __all_sync(0xFFFFFFFFu,
+                                    cluster_wait(bar_in_full, uint32_t(local & 1), abort, p.status, 12, p.wait_limit));
+                    const uint8_t *const xb = smem + (rank ? kSmInbox : kSmOwn),
+                                  *const yb = smem + (rank ? kSmOwn : kSmInbox);
+                    const int i0 = it.base + kTile + 64 * rank;
+#pragma unroll 1
+                    for (int e = e0; ok && e < e1; ++e) {
+                        const int c0 = 16 * (e >> 2), j = 32 * (e & 3) + lane;
+                        if (i0 + c0 >= n_in) break;
+                        uint32_t xr[16];
+                        float yv[16];
+                        const int o = c0 * kHalfPitch + j * 4;
+#pragma unroll
+                        for (int k = 0; k < 16; ++k) {
+                            xr[k] = *reinterpret_cast<const uint32_t *>(xb + o + k * kHalfPitch);
+                            yv[k] = *reinterpret_cast<const float *>(yb + o + k * kHalfPitch);
+                        }
+                        emit16(i0 + c0, it.base + j, xr, yv, i0 + c0 + 15 < n_in);
+                    }
                 }
-            };
-            if (!kPair) {
-                release_tmem();
-                named_sync(2, kEpiWarps * 32);             // the diagonal tile's rows have been read
-                continue;
+                // every read of the inbox has returned (its values have been used)
+                __syncwarp();
+                if (ok && lane == 0) remote_arrive(map_rank(bar_in_free, uint32_t(rank ^ 1)));
             }
-            if (rank == 1) {
-                named_sync(2, kEpiWarps * 32);             // the diagonal tile's rows have been read
-                if (q >= 2) put_row(il, 0, kTile);
-                release_tmem();
-            }
-            ok = agree(cluster_wait(bar_in_full, uint32_t(local & 1), abort, p.status, 12, p.wait_limit));
-            if (!ok) break;
-            if (rank == 1) {
-                emit(t0, it.base, 64, kTile, 64, smem + kSmXch + 64 * kXchPitch, 0, true, false);
-            } else {
-                emit(t0 + kTile, it.base, 0, 64, 0, smem + kSmInbox, kTile, false, false);
-                release_tmem();
-            }
-            // every read of the inbox has returned (its values have been used)
-            remote_arrive(map_rank(bar_in_free, uint32_t(rank ^ 1)));
-            if (rank == 1) named_sync(2, kEpiWarps * 32);  // the off-diagonal rows have been read
+            // the next item's vote follows every read of the buffers; a failed wait shows in it
+            if (!ok && item + item_step < p.n_items) agree(false);
         }
         // after a timeout, rows may still be on their way to the pair's inbox
         if (kPair && !ok) __nanosleep(100000);
