@@ -148,4 +148,28 @@ int set_last_error(int status);
 cudaError_t launch_dump(const int32_t *acc, int32_t *vis, size_t n_words, bool fresh,
                         cudaStream_t s, int *launches);
 
+// Programmatic overlap of the launches of one call: the first of these lets the next
+// launch's CTAs take the SMs as this one's leave them (once all of its CTAs have got there
+// or ended); the second waits until the launch before has ended and its writes are there.
+__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;"); }
+__device__ __forceinline__ void wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Launch with the attribute that `overlap` asks for.
+template <typename... Args>
+cudaError_t launch_overlapping(void (*fn)(Args...), int grid, int threads, size_t smem, bool overlap, cudaStream_t s,
+                               const Args &...args)
+{
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(unsigned(grid));
+    cfg.blockDim = dim3(unsigned(threads));
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, fn, args...);
+}
+
 }  // namespace corr

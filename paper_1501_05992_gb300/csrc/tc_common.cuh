@@ -350,13 +350,6 @@ __device__ __forceinline__ uint32_t imad(uint32_t a, uint32_t b, uint32_t c)
     return d;
 }
 
-// The launches of one call write disjoint parts of the output and may overlap: each
-// lets the next one's CTAs take the SMs as its own leave them (in place of an empty
-// last round per launch: 384 inputs x 384 channels x 5000 samples 0.51 -> 0.45 ms, 1024 x
-// 128 x 10000 1.81 -> 1.74 ms), and ends only when the one before has.
-__device__ __forceinline__ void let_next_launch_start() { asm volatile("griddepcontrol.launch_dependents;"); }
-__device__ __forceinline__ void wait_for_launch_before() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-
 // TMEM allocation by one warp (kPair: of both CTAs of a pair); the address goes to `slot`.
 template <bool kPair>
 __device__ __forceinline__ void tmem_alloc(uint32_t slot, uint32_t cols)
@@ -393,23 +386,5 @@ cudaError_t launch_xeng_tile(const TcArray *arrays, int count, bool fresh, bool 
 // maps[k] is array k's tensor map (boxes of 128 inputs x 1 channel x 32 samples).
 cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int count, bool fresh, bool zero_invalid,
                             int dev, DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
-
-// Launch with the attribute that `overlap` asks for.
-template <typename... Args>
-cudaError_t launch_overlapping(void (*fn)(Args...), int grid, int threads, size_t smem, bool overlap, cudaStream_t s,
-                               const Args &...args)
-{
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(unsigned(grid));
-    cfg.blockDim = dim3(unsigned(threads));
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr{};
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = overlap ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, fn, args...);
-}
 
 }  // namespace corr

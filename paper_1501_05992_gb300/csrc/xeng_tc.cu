@@ -63,6 +63,10 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
 
 // The launches of the arrays of one mode, longest integrations first (a CTA's
 // last items are then its shortest).
+// The launches of one call write disjoint parts of the output and may overlap: each lets
+// the next one's CTAs take the SMs as its own leave them (in place of an empty last round
+// per launch: 384 inputs x 384 channels x 5000 samples 0.51 -> 0.45 ms, 1024 x 128 x 10000
+// 1.81 -> 1.74 ms), and ends only when the one before has.
 cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero_invalid, int dev,
                          DeviceStatus *status, const TcOptions &opt, cudaStream_t s, int *launches)
 {
