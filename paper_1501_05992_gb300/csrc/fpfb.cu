@@ -17,7 +17,9 @@
 // Work decomposition.  A CTA of 4 warps takes 16 consecutive inputs of one
 // coarse channel over one group of frames (more on very long inputs): G = 8, inputs in
 // sub-batches of 2, so that one unit (group, sub-batch) is 16 (frame, input)
-// transforms, taken in three phases separated by CTA barriers.
+// transforms, taken in three phases separated by barriers: of the two warps that share
+// an input of the sub-batch, so that the CTA's two pairs of warps drift apart and fill each
+// other's waits, or of the CTA where spectra are stored.
 //
 //  1. Windowing.  Warp w takes input w / 2 of the sub-batch and the points
 //     64 (w mod 2) .. + 63, lane l the pair of points (2 l, 2 l + 1) of that
@@ -37,7 +39,7 @@
 //     the two halves of its float pairs (adjacent points: one 8-byte load per
 //     pair), does the 8-point DFT over n2 in registers and applies
 //     W128^{n1 k2} (a shared-memory table).
-//  3. 16-point DFTs.  A thread takes one transform and one k2: its 16 values
+//  3. 16-point DFTs.  A thread takes one transform (of its pair's eight) and one k2: its 16 values
 //     over n1 arrive as 8 float pairs (even n1, odd n1), so the two 8-point
 //     DFTs of the even and odd halves are paired instructions and the last
 //     radix-2 step (W16^{k1}) is scalar.  The 16 outputs are clamped, rounded
@@ -46,6 +48,10 @@
 //     one fine channel, the CTA's 16 inputs: 16 bytes) is written with one
 //     16-byte store.  Scattered stores of a few bytes per row cost the store
 //     path one transaction each, which is why a CTA gathers 16 inputs.
+//
+// Codes of 24 coarse channels x 256 inputs x 500 frames: 0.979 -> 0.911 ms with
+// barriers of two warps and their stores spread over the banks (0.927 without the
+// former, 0.941 without the latter) and one test per unit for the blocks it loads.
 //
 // No lane exchanges data with another through shuffles: the two transposes
 // go through shared memory, laid out so that every access takes the minimum
@@ -159,10 +165,19 @@ __device__ __forceinline__ void dft8(C2 (&x)[8])
     dft4(x[4], x[5], x[6], x[7]);
 }
 
-template <int NB>
+// kWhole: test once whether all blocks are there instead of one by one (codes of 24 coarse
+// channels x 256 inputs x 500 frames 0.979 -> 0.938 ms; the kernels that write spectra
+// lose by it, 12 x 256 x 300 1.34 -> 1.39 ms).
+template <bool kWhole, int NB>
 __device__ __forceinline__ void load_blocks(uint32_t (&w)[NB], const int8_t *x, long long b0, long long n_blocks,
                                             bool active)
 {
+    if (kWhole && active && b0 + NB <= n_blocks) {
+        const int8_t *const at = x + b0 * (2 * kPfbPoints);
+#pragma unroll
+        for (int bb = 0; bb < NB; ++bb) w[bb] = *reinterpret_cast<const uint32_t *>(at + bb * (2 * kPfbPoints));
+        return;
+    }
 #pragma unroll
     for (int bb = 0; bb < NB; ++bb) {
         const long long b = b0 + bb;
@@ -196,6 +211,9 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
     // (Re pair, Im pair) per (k2, r); times the code scale when only codes are
     // written, the scale then riding on the twiddles
     constexpr bool kFold = kVolt && !kSpec;
+    // bytes by which a row of codes is rotated per channel: 4 spread a warp's byte stores
+    // (8 frames x 4 channels) over the banks
+    constexpr int kRotate = kSpec ? 0 : 4;
     const float tws = kFold ? a.scale : 1.0f;
     if (threadIdx.x < 64) {
         const int k2 = threadIdx.x >> 3, r = threadIdx.x & 7;
@@ -214,7 +232,13 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
     // the blocks of the first unit (group, sub-batch); every unit loads those
     // of the next one before its transforms, so that the loads complete behind them
     uint32_t wblk[B];
-    load_blocks(wblk, stream(0), m0, n_blocks, i0 + iw < a.N);
+    // the threads that exchange a unit's data: the two warps of an input, or (where spectra
+    // are stored, whose pairs of inputs lie side by side) the CTA
+    auto sync_team = [&] {
+        if (kSpec) __syncthreads();
+        else asm volatile("bar.sync %0, 64;" ::"r"(1 + iw) : "memory");
+    };
+    load_blocks<!kSpec>(wblk, stream(0), m0, n_blocks, i0 + iw < a.N);
     __syncthreads();
 
     for (int g0 = m0; g0 < m1; g0 += G) {
@@ -255,10 +279,10 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                 const bool more = sb + 1 < n_sub;
                 if (more || g0 + G < m1) {
                     const int nsb = more ? sb + 1 : 0;
-                    load_blocks(wblk, stream(nsb), more ? g0 : g0 + G, n_blocks, i0 + nsb * kPfbSub + iw < a.N);
+                    load_blocks<!kSpec>(wblk, stream(nsb), more ? g0 : g0 + G, n_blocks, i0 + nsb * kPfbSub + iw < a.N);
                 }
             }
-            __syncthreads();
+            sync_team();
             // ---- 2. 8-point DFTs over n2 (transform t / 8, columns n1 = 2 r, 2 r + 1)
             {
                 const int xf = threadIdx.x >> 3, r = threadIdx.x & 7;
@@ -288,10 +312,11 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                     z[k2 * 8 + (r ^ k2)] = make_float4(v.r.x, v.r.y, v.i.x, v.i.y);
                 }
             }
-            __syncthreads();
-            // ---- 3. 16-point DFTs over n1 (warp k2, lane = transform)
+            sync_team();
+            // ---- 3. 16-point DFTs over n1
             {
-                const int xf = lane & 15, k2 = 2 * warp + (lane >> 4);
+                const int xf = kSpec ? lane & 15 : iw * G + (lane & 7),
+                          k2 = kSpec ? 2 * warp + (lane >> 4) : 4 * (warp & 1) + (lane >> 3);
                 const float4 *z = reinterpret_cast<const float4 *>(Z + xf * kZStride) + k2 * 8;
                 C2 e[8];                        // .x: n1 = 2 r (even), .y: n1 = 2 r + 1 (odd)
 #pragma unroll
@@ -337,7 +362,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                             const float2 s = kFold ? make_float2(yr, yi) : mul2(make_float2(yr, yi), dup2(a.scale));
                             const float2 w = add2(make_float2(fminf(fmaxf(s.x, -7.0f), 7.0f),
                                                               fminf(fmaxf(s.y, -7.0f), 7.0f)), dup2(12582920.0f));
-                            tile[f * kTileFrame + c * kPfbInputs + sb * kPfbSub + iw3] =
+                            tile[f * kTileFrame + c * kPfbInputs + ((sb * kPfbSub + iw3 + kRotate * k2) & 15)] =
                                 uint8_t(__float_as_uint(w.x) * 16u + __float_as_uint(w.y));
                         }
                     }
@@ -348,7 +373,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
             // first barrier (every 16-point load of this unit comes before it)
         }
         if (kVolt) {
-            // ---- 4. the group's codes, one 32-byte row piece (32 inputs) per output row
+            // ---- 4. the group's codes, one 16-byte row piece (16 inputs) per output row
             __syncthreads();
             const int nf = min(G, m1 - g0);
             const bool full = i0 + kPfbInputs <= a.N && (a.N & 15) == 0 &&
@@ -360,17 +385,18 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                 const uint8_t *src = tile + f * kTileFrame + c * kPfbInputs + 16 * hh;
                 if (full) {
                     uint4 v = *reinterpret_cast<const uint4 *>(src);
+                    if (kRotate && (c & 1)) v = make_uint4(v.y, v.z, v.w, v.x);
+                    if (kRotate && (c & 2)) v = make_uint4(v.z, v.w, v.x, v.y);
                     v.x ^= 0x88888888u;
                     v.y ^= 0x88888888u;
                     v.z ^= 0x88888888u;
                     v.w ^= 0x88888888u;
                     *reinterpret_cast<uint4 *>(dst) = v;
                 } else {
-                    for (int w = 0; w < 16 && i0 + 16 * hh + w < a.N; ++w) dst[w] = src[w] ^ 0x88u;
+                    for (int w = 0; w < 16 && i0 + 16 * hh + w < a.N; ++w) dst[w] = src[(w + kRotate * c) & 15] ^ 0x88u;
                 }
             }
-            // the next group writes the codes only after two more barriers,
-            // which every thread reaches after its copy-out
+            if (g0 + G < m1) __syncthreads();          // before the next group's codes
         }
     }
 }
