@@ -14,12 +14,12 @@
 // the X-engine's input layout [frame][q * 128 + c][input], so the F and X
 // stages chain on the device.
 //
-// Work decomposition.  A CTA of 4 warps takes 16 consecutive inputs of one
-// coarse channel over one group of frames (more on very long inputs): G = 8, inputs in
-// sub-batches of 2, so that one unit (group, sub-batch) is 16 (frame, input)
-// transforms, taken in three phases separated by barriers: of the two warps that share
-// an input of the sub-batch, so that the CTA's two pairs of warps drift apart and fill each
-// other's waits, or of the CTA where spectra are stored.
+// Work decomposition.  A CTA takes 16 consecutive inputs of one coarse channel over
+// one group of frames (more on very long inputs): G = 8, inputs in sub-batches of 2 (4 where
+// spectra are stored) with two warps each, so that one unit (group, sub-batch) is 16
+// (32) (frame, input) transforms, taken in three phases separated by barriers: of the two
+// warps that share an input of the sub-batch, so that a CTA's pairs of warps drift apart
+// and fill each other's waits, or of the CTA where spectra are stored.
 //
 //  1. Windowing.  Warp w takes input w / 2 of the sub-batch and the points
 //     64 (w mod 2) .. + 63, lane l the pair of points (2 l, 2 l + 1) of that
@@ -39,15 +39,18 @@
 //     the two halves of its float pairs (adjacent points: one 8-byte load per
 //     pair), does the 8-point DFT over n2 in registers and applies
 //     W128^{n1 k2} (a shared-memory table).
-//  3. 16-point DFTs.  A thread takes one transform (of its pair's eight) and one k2: its 16 values
-//     over n1 arrive as 8 float pairs (even n1, odd n1), so the two 8-point
+//  3. 16-point DFTs.  A thread takes one transform and one k2: its 16 values over n1 arrive
+//     as 8 float pairs (even n1, odd n1), so the two 8-point
 //     DFTs of the even and odd halves are paired instructions and the last
 //     radix-2 step (W16^{k1}) is scalar.  The 16 outputs are clamped, rounded
 //     and packed into codes in a shared-memory tile of the CTA's 16 inputs.
 //  4. After the last sub-batch of a group, each output row piece (one frame,
 //     one fine channel, the CTA's 16 inputs: 16 bytes) is written with one
 //     16-byte store.  Scattered stores of a few bytes per row cost the store
-//     path one transaction each, which is why a CTA gathers 16 inputs.
+//     path one transaction each, which is why a CTA gathers 16 inputs.  Spectra go out
+//     from phase 3, four inputs (32 bytes, a whole sector) side by side: half sectors
+//     of two inputs left L2 before they met, 12 coarse channels x 256 inputs x 300 frames
+//     1.34 ms against 0.51 (0.60 with eight inputs, one CTA per SM).
 //
 // Codes of 24 coarse channels x 256 inputs x 500 frames: 0.979 -> 0.911 ms with
 // barriers of two warps and their stores spread over the banks (0.927 without the
@@ -67,12 +70,16 @@ namespace corr {
 namespace {
 
 constexpr int kPfbPoints = 128;
-constexpr int kPfbThreads = 128;              // 4 warps
-constexpr int kPfbSub = 2;                    // inputs per sub-batch, two windowing warps each
-constexpr int kPfbInputs = 16;                // inputs per CTA: 8 sub-batches
+constexpr int kPfbInputs = 16;                // inputs per CTA, in sub-batches
 constexpr int kPfbGroup = 8;                  // frames per group
-constexpr int kPfbXf = kPfbSub * kPfbGroup;   // transforms per unit
-constexpr int kPfbCtasPerSm = 4;
+// inputs per sub-batch, with two warps each
+template <bool kSpec>
+constexpr int kPfbSub = kSpec ? 4 : 2;
+template <bool kSpec>
+constexpr int kPfbThreads = 64 * kPfbSub<kSpec>;
+template <bool kSpec>
+constexpr int kPfbXf = kPfbSub<kSpec> * kPfbGroup;   // transforms per unit
+constexpr int kPfbThreadsPerSm = 512;
 // shared memory: windowed frames [16][Re 128 | Im 128 | pad 16] floats (the
 // pad spreads the transforms over the banks), 8-point results [16 transforms]
 // [8 k2 rows of 8 float4 | pad 16 bytes], the W128 twiddles [8 k2][8 r]
@@ -81,7 +88,8 @@ constexpr int kPfbCtasPerSm = 4;
 constexpr int kUStride = 2 * kPfbPoints + 16;             // floats
 constexpr int kZStride = 8 * 8 * 4 + 4;                   // floats
 constexpr int kTileFrame = kPfbPoints * kPfbInputs + 16;  // bytes
-constexpr size_t kPfbSmem = sizeof(float) * (kPfbXf * kUStride + kPfbXf * kZStride + 8 * 8 * 4) +
+template <bool kSpec>
+constexpr size_t kPfbSmem = sizeof(float) * (kPfbXf<kSpec> * (kUStride + kZStride) + 8 * 8 * 4) +
                             size_t(kPfbGroup) * kTileFrame;
 
 struct PfbArgs {
@@ -165,14 +173,13 @@ __device__ __forceinline__ void dft8(C2 (&x)[8])
     dft4(x[4], x[5], x[6], x[7]);
 }
 
-// kWhole: test once whether all blocks are there instead of one by one (codes of 24 coarse
-// channels x 256 inputs x 500 frames 0.979 -> 0.938 ms; the kernels that write spectra
-// lose by it, 12 x 256 x 300 1.34 -> 1.39 ms).
-template <bool kWhole, int NB>
+// One test whether all blocks are there, before one by one (codes of 24 coarse channels x
+// 256 inputs x 500 frames 0.979 -> 0.938 ms).
+template <int NB>
 __device__ __forceinline__ void load_blocks(uint32_t (&w)[NB], const int8_t *x, long long b0, long long n_blocks,
                                             bool active)
 {
-    if (kWhole && active && b0 + NB <= n_blocks) {
+    if (active && b0 + NB <= n_blocks) {
         const int8_t *const at = x + b0 * (2 * kPfbPoints);
 #pragma unroll
         for (int bb = 0; bb < NB; ++bb) w[bb] = *reinterpret_cast<const uint32_t *>(at + bb * (2 * kPfbPoints));
@@ -186,20 +193,21 @@ __device__ __forceinline__ void load_blocks(uint32_t (&w)[NB], const int8_t *x, 
 }
 
 template <int TAPS, bool kSpec, bool kVolt>
-__global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArgs a)
+__global__ void __launch_bounds__(kPfbThreads<kSpec>, kPfbThreadsPerSm / kPfbThreads<kSpec>)
+fpfb_kernel(PfbArgs a)
 {
-    constexpr int G = kPfbGroup;
+    constexpr int G = kPfbGroup, kSub = kPfbSub<kSpec>, kXf = kPfbXf<kSpec>, kThreads = kPfbThreads<kSpec>;
     constexpr int B = G + TAPS - 1;             // blocks that feed a group
     extern __shared__ __align__(16) float smem[];
-    float *const U = smem;                                    // [32][kUStride]
-    float *const Z = U + kPfbXf * kUStride;                   // [32][kZStride]
-    float4 *const TW = reinterpret_cast<float4 *>(Z + kPfbXf * kZStride);   // [8][8]
+    float *const U = smem;                                    // [kXf][kUStride]
+    float *const Z = U + kXf * kUStride;                   // [kXf][kZStride]
+    float4 *const TW = reinterpret_cast<float4 *>(Z + kXf * kZStride);   // [8][8]
     uint8_t *const tile = reinterpret_cast<uint8_t *>(TW + 8 * 8);          // [G][kTileFrame]
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int q = blockIdx.z;
     const int i0 = blockIdx.x * kPfbInputs;
-    const int n_sub = min(kPfbInputs, a.N - i0 + kPfbSub - 1) / kPfbSub;   // sub-batches with an input
+    const int n_sub = min(kPfbInputs, a.N - i0 + kSub - 1) / kSub;   // sub-batches with an input
     const int iw = warp >> 1;                   // windowing: this warp's input of a sub-batch, and half
     const int p0 = 64 * (warp & 1) + 2 * lane;
     const int m0 = blockIdx.y * a.fpc;
@@ -212,7 +220,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
     // written, the scale then riding on the twiddles
     constexpr bool kFold = kVolt && !kSpec;
     // bytes by which a row of codes is rotated per channel: 4 spread a warp's byte stores
-    // (8 frames x 4 channels) over the banks
+    // over the banks (codes only: 8 frames x 4 channels of one input)
     constexpr int kRotate = kSpec ? 0 : 4;
     const float tws = kFold ? a.scale : 1.0f;
     if (threadIdx.x < 64) {
@@ -226,19 +234,19 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
     for (int p = 0; p < TAPS; ++p) h2[p] = *reinterpret_cast<const float2 *>(a.h + p * kPfbPoints + p0);
     const float2 bias = dup2(-8388736.0f);
     auto stream = [&](int sb) {                 // this warp's input stream in sub-batch sb
-        const int i = i0 + sb * kPfbSub + iw;
+        const int i = i0 + sb * kSub + iw;
         return a.x + (size_t(q) * a.N + (i < a.N ? i : 0)) * size_t(a.S) * 2 + 2 * p0;
     };
     // the blocks of the first unit (group, sub-batch); every unit loads those
     // of the next one before its transforms, so that the loads complete behind them
     uint32_t wblk[B];
     // the threads that exchange a unit's data: the two warps of an input, or (where spectra
-    // are stored, whose pairs of inputs lie side by side) the CTA
+    // are stored, a warp's lanes over several inputs) the CTA
     auto sync_team = [&] {
         if (kSpec) __syncthreads();
         else asm volatile("bar.sync %0, 64;" ::"r"(1 + iw) : "memory");
     };
-    load_blocks<!kSpec>(wblk, stream(0), m0, n_blocks, i0 + iw < a.N);
+    load_blocks(wblk, stream(0), m0, n_blocks, i0 + iw < a.N);
     __syncthreads();
 
     for (int g0 = m0; g0 < m1; g0 += G) {
@@ -279,7 +287,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                 const bool more = sb + 1 < n_sub;
                 if (more || g0 + G < m1) {
                     const int nsb = more ? sb + 1 : 0;
-                    load_blocks<!kSpec>(wblk, stream(nsb), more ? g0 : g0 + G, n_blocks, i0 + nsb * kPfbSub + iw < a.N);
+                    load_blocks(wblk, stream(nsb), more ? g0 : g0 + G, n_blocks, i0 + nsb * kSub + iw < a.N);
                 }
             }
             sync_team();
@@ -315,8 +323,9 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
             sync_team();
             // ---- 3. 16-point DFTs over n1
             {
-                const int xf = kSpec ? lane & 15 : iw * G + (lane & 7),
-                          k2 = kSpec ? 2 * warp + (lane >> 4) : 4 * (warp & 1) + (lane >> 3);
+                // codes: a warp pair's own input; spectra: a warp's lanes over 4 inputs
+                const int xf = kSpec ? threadIdx.x % kXf : iw * G + (lane & 7),
+                          k2 = kSpec ? threadIdx.x / kXf : 4 * (warp & 1) + (lane >> 3);
                 const float4 *z = reinterpret_cast<const float4 *>(Z + xf * kZStride) + k2 * 8;
                 C2 e[8];                        // .x: n1 = 2 r (even), .y: n1 = 2 r + 1 (odd)
 #pragma unroll
@@ -326,7 +335,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                     e[r].i = make_float2(v.z, v.w);
                 }
                 dft8(e);                        // E[k] (.x) and O[k] (.y): k even in e[k / 2], odd in e[4 + k / 2]
-                const int iw3 = xf / G, f = xf % G, m = g0 + f, i = i0 + sb * kPfbSub + iw3;
+                const int iw3 = xf / G, f = xf % G, m = g0 + f, i = i0 + sb * kSub + iw3;
                 // Y[k2 + 8 k1] = E[k1] + W16^{k1} O[k1], Y[k2 + 8 (k1 + 8)] = E[k1] - W16^{k1} O[k1]
                 const float c16 = 0.92387953251128674f, s16 = 0.38268343236508977f, h = 0.70710678118654752f;
                 const float wre[8] = {1.0f, c16, h, s16, 0.0f, -s16, -h, -c16};
@@ -362,7 +371,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
                             const float2 s = kFold ? make_float2(yr, yi) : mul2(make_float2(yr, yi), dup2(a.scale));
                             const float2 w = add2(make_float2(fminf(fmaxf(s.x, -7.0f), 7.0f),
                                                               fminf(fmaxf(s.y, -7.0f), 7.0f)), dup2(12582920.0f));
-                            tile[f * kTileFrame + c * kPfbInputs + ((sb * kPfbSub + iw3 + kRotate * k2) & 15)] =
+                            tile[f * kTileFrame + c * kPfbInputs + ((sb * kSub + iw3 + kRotate * k2) & 15)] =
                                 uint8_t(__float_as_uint(w.x) * 16u + __float_as_uint(w.y));
                         }
                     }
@@ -379,7 +388,7 @@ __global__ void __launch_bounds__(kPfbThreads, kPfbCtasPerSm) fpfb_kernel(PfbArg
             const bool full = i0 + kPfbInputs <= a.N && (a.N & 15) == 0 &&
                               (reinterpret_cast<uintptr_t>(a.volt) & 15) == 0;
             constexpr int kChunks = kPfbInputs / 16;
-            for (int t = threadIdx.x; t < nf * kPfbPoints * kChunks; t += kPfbThreads) {
+            for (int t = threadIdx.x; t < nf * kPfbPoints * kChunks; t += kThreads) {
                 const int row = t / kChunks, hh = t % kChunks, f = row / kPfbPoints, c = row % kPfbPoints;
                 uint8_t *dst = a.volt + (size_t(g0 + f) * C + size_t(q) * kPfbPoints + c) * a.N + i0 + 16 * hh;
                 const uint8_t *src = tile + f * kTileFrame + c * kPfbInputs + 16 * hh;
@@ -412,14 +421,14 @@ cudaError_t launch_pfb(const PfbArgs &a, dim3 grid, int dev, cudaStream_t s)
     static bool configured[kPfbMaxDevices] = {};
     if (dev >= kPfbMaxDevices || !configured[dev]) {
         cudaError_t e = cudaFuncSetAttribute(fpfb_kernel<TAPS, kSpec, kVolt>,
-                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPfbSmem));
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, int(kPfbSmem<kSpec>));
         if (e == cudaSuccess)
             e = cudaFuncSetAttribute(fpfb_kernel<TAPS, kSpec, kVolt>,
                                      cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         if (e != cudaSuccess) return e;
         if (dev < kPfbMaxDevices) configured[dev] = true;
     }
-    fpfb_kernel<TAPS, kSpec, kVolt><<<grid, kPfbThreads, kPfbSmem, s>>>(a);
+    fpfb_kernel<TAPS, kSpec, kVolt><<<grid, kPfbThreads<kSpec>, kPfbSmem<kSpec>, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -449,7 +458,7 @@ cudaError_t launch_fine_pfb(const int8_t *x, int n_coarse, int n_inputs, long lo
     // frames per CTA: one group, as long as the grid allows it.  A CTA's prologue (the
     // window, the twiddles, the first loads) hides behind the SM's other CTAs, while
     // runs of up to 120 frames left the last CTAs' SMs idle: 24 coarse channels x 256
-    // inputs x 500 frames 1.07 -> 0.98 ms, 12 x 256 x 300 with spectra 1.49 -> 1.34 ms.
+    // inputs x 500 frames 1.07 -> 0.98 ms, 12 x 256 x 300 with spectra (then) 1.49 -> 1.34 ms.
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;

@@ -1,6 +1,6 @@
-"""Fine filterbank, codes only: inputs so long that a CTA takes several groups of
-frames give the codes of their pieces, which take one group per CTA; and the codes
-of whole and ragged sets of 16 inputs are those of the inputs taken alone."""
+"""Fine filterbank: inputs so long that a CTA takes several groups of frames give the
+codes of their pieces, which take one group per CTA; and the codes and spectra of
+whole and ragged sets of inputs are those of the inputs taken alone."""
 import pytest
 import torch
 
@@ -36,3 +36,17 @@ def test_inputs_by_themselves(n):
     got = _codes(x, h)
     for i in {0, 1, n // 2, n - 1}:
         assert torch.equal(got[:, :, i], _codes(x[:, i:i + 1].contiguous(), h)[:, :, 0])
+
+
+@pytest.mark.parametrize("volt", [False, True])
+@pytest.mark.parametrize("n", [2, 3, 4, 5, 15, 16, 18, 33])
+@pytest.mark.parametrize("taps,frames", [(12, 3), (12, 20), (1, 17)])
+def test_spectra_by_themselves(n, taps, frames, volt):
+    h = torch.from_numpy(coarse.kaiser_sinc_window(12)[:128 * taps]).float().cuda()
+    x = torch.from_numpy(coarse.coarse_samples(n, 2, n, 128 * (frames + taps - 1))).cuda()
+    codes, spec = corr.fine_pfb(x, h, 0.01, volt=volt, spec=True)
+    for i in {0, 1, n // 2, n - 1}:
+        one_codes, one_spec = corr.fine_pfb(x[:, i:i + 1].contiguous(), h, 0.01, volt=volt, spec=True)
+        assert torch.equal(spec[:, :, i], one_spec[:, :, 0])
+        if volt:
+            assert torch.equal(codes[:, :, i], one_codes[:, :, 0])
