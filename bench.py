@@ -47,7 +47,7 @@ WORKLOADS = {
     "coarse_channel": ([(256, 128, 5000)], 1, 1502),
     # one integration of the full band (3.9 GB of voltages): a small case for traffic captures
     "integration": ([(256, 3072, 5000)], 1, 1503),
-    # a quarter of the band, one integration (1 GB of voltages, 1536 items: about ten per CTA, so
+    # a quarter of the band, one integration (1 GB of voltages, 768 items: about ten per CTA pair, so
     # the steady state rather than the tail): a small case for full profiles
     "quarter_band": ([(256, 768, 5000)], 1, 1507),
     "uneven_batch": ([(128, 1536, 2000), (256, 3072, 5000), (1024, 512, 10000)], 1, 1504),
@@ -597,7 +597,7 @@ def measure_uneven_batch(stream_, dev, peaks, sm_count):
     res.update({"ms_batch": ms_all, "value": cmac_all / (ms_all * 1e-3), "unit": "CMAC/s",
                 "achieved": roof["achieved"], "peak": roof["peak"], "frac": roof["frac"],
                 "exact": all(x["exact"] and x["same_as_in_batch"] for x in res["arrays"]),
-                "launch": "one corr_batch_integrate: the tensor-core arrays share one persistent launch"})
+                "launch": "one corr_batch_integrate: the tensor-core arrays share its persistent launches"})
     batch.close()
     del volts, outs
     return res
@@ -830,11 +830,11 @@ def run_ours(args, world, rank, local):
     avg_ms = xe_ms / max(1, xe_timed)
     main_path = paths[max(range(len(arrays)), key=lambda a: arrays[a][0] ** 2 * arrays[a][1] * arrays[a][2])]
     roof = roofline_for(main_path, ops_per_launch, avg_ms, peaks, src, sm_count, measured_probes(dev))
-    roof["traffic"] = (measured_traffic(os.path.join(ROOT, "paper_1501_05992_gb300", "csrc", "xeng_tc.cu"),
-                                        os.path.join(ROOT, "profiles", "xeng_tc_full_band_traffic.md"),
+    roof["traffic"] = (measured_traffic(os.path.join(ROOT, "paper_1501_05992_gb300", "csrc", "xeng_diag.cuh"),
+                                        os.path.join(ROOT, "profiles", "xeng_pair_full_band_traffic.md"),
                                         args.workload) if main_path == "tc_fp8" else None)
     roof["kernel"] = {"cudacore": "xeng_dp4a_kernel", "mma_i8": "xeng_mma8_kernel",
-                      "tc_fp8": "xeng_tc_kernel"}[main_path]
+                      "tc_fp8": "xeng_pair_kernel"}[main_path]
     roof["launches_per_step"] = xe_per_step
     roof["avg_launch_ms"] = avg_ms
     roof["timing"] = timing_note

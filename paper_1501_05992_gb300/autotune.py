@@ -5,11 +5,9 @@ candidate (path, tile) the device supports is timed on a probe block of the
 same N and T (random bytes: the kernels' speed does not depend on the values)
 with a bounded number of channels, and the fastest is kept in a JSON cache
 keyed by device name and shape.  The candidates are the library's tile shapes
-(Section 3.4.2: the tile sets the arithmetic intensity): tcgen05 FP8 with
-every work item one 128 x 128 tile pair (tile 128; each item's epilogue
-overlaps the next item's MMAs) or with pair items, a diagonal tile and the
-tile left of it as one 256-row column sharing one conversion (tile 256);
-int8 mma.sync on 64 x 64; and the dp4a CUDA-core kernel on 64 x 64 or
+(Section 3.4.2: the tile sets the arithmetic intensity): tcgen05 FP8, whose
+split into tiles is by shape (128 and 256 measure the same kernels); int8
+mma.sync on 64 x 64; and the dp4a CUDA-core kernel on 64 x 64 or
 32 x 32 tiles.
 """
 from __future__ import annotations

@@ -229,9 +229,9 @@ class Correlator:
         return PATH_NAMES[self._lib.corr_get_path(self._ctx)]
 
     def set_tile(self, tile: int) -> None:
-        """Tile shape (corr_set_tile): 32 or 64 for the CUDA-core path, 128
-        (single tile-pair items) or 256 (pair items) for the tcgen05 path,
-        0 to choose by shape."""
+        """Tile shape (corr_set_tile): 32 or 64 for the CUDA-core path, 0 to
+        choose by shape; 128 and 256 are accepted for the tcgen05 path, whose
+        split into tiles is always by shape."""
         _check(self._lib.corr_set_tile(self._ctx, int(tile)), f"corr_set_tile({tile})")
 
     def set_wait_limit(self, cycles: int) -> None:
@@ -392,8 +392,8 @@ class Graph:
 
 
 class Batch:
-    """Several arrays correlated together; tensor-core arrays share one
-    persistent launch.  ``arrays`` holds (n_inputs, n_chan, n_time_per_int)
+    """Several arrays correlated together; tensor-core arrays share
+    persistent launches.  ``arrays`` holds (n_inputs, n_chan, n_time_per_int)
     tuples or dicts with those keys plus optional ``path`` / ``zero_invalid``."""
 
     def __init__(self, arrays, device: torch.device | int | None = None):

@@ -17,9 +17,9 @@
 // Both are HBM-bound: one byte read and 4 (words: 2 planes x 2 bytes) or 2
 // (K-major) bytes written per complex sample.
 //
-// The tensor-core path reads the packed bytes themselves, through TMA, which
-// needs rows (the n inputs of one channel and sample) that start on 16-byte
-// boundaries.  For other input counts the rows are first copied to a stride
+// The tensor-core path reads the packed bytes themselves.  Beyond 256 inputs they come
+// through TMA, which needs rows (the n inputs of one channel and sample) that start on
+// 16-byte boundaries.  For other input counts the rows are first copied to a stride
 // of round_up(n, 16) bytes (the bytes between rows are never read: the
 // tensor map's extent is n and TMA fills columns past it with zeros).
 #include "decode.cuh"

@@ -41,8 +41,8 @@
 // samples) it takes 1.30-1.37 ms, against 1.68-1.78 ms for a kernel of 128-input tiles
 // in [Re | Im] form, at the card's 1400 W; the MMAs alone take 1.05 ms at the same
 // power and the converters alone 0.71 ms at 585 W, so what counts is work per
-// integration: MMAs (two thirds of that kernel's) and instructions.  The
-// shared-memory pipe is 70 % busy, the tensor pipe 63 %, the ALU pipe 50 %.  Short
+// integration: MMAs (two thirds of that kernel's) and instructions.  The tensor
+// pipe is 67 % busy, the ALU pipe 52 % (a quarter of the band).  Short
 // launches are bound by the epilogue's exchange and stores (adding 500 samples to the
 // full band's triangle: 0.38 ms, of which 0.28 ms is what the adds alone take in L2).  One tile
 // alone is bound by its MMAs (M=128 N=128 reads 8 KB of operands in 64 cycles) and

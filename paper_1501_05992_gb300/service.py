@@ -15,8 +15,8 @@ are integrated on the GPU for an operator-chosen time before being copied out
   are rejected with ``CORR_E_BUDGET``;
 * a dispatcher gathers the blocks that have arrived (at most one per array per
   tick), copies them into the arrays' device rings on a copy stream and
-  correlates them with one batched call (tensor-core arrays share one
-  persistent launch); every ``blocks_per_dump`` blocks an array's integration
+  correlates them with one batched call (tensor-core arrays share
+  persistent launches); every ``blocks_per_dump`` blocks an array's integration
   is dumped and copied to pinned host memory;
 * sequence numbers are checked: a missing block is counted and the
   integration it belonged to is flagged (no unsynchronised data are merged

@@ -34,3 +34,25 @@ def test_stream_ends(lane, offset, count):
     want_v, want_c = oracle.ingest(sel, 9)
     assert np.array_equal(cnt.cpu().numpy().astype(np.int64), want_c)
     assert np.array_equal(volt.cpu().numpy(), want_v)
+
+
+def test_capture(lane):
+    """The call's three launches, which overlap, replayed from a graph on new packets."""
+    sel = lane[:4003]
+    p = torch.from_numpy(np.ascontiguousarray(sel)).cuda()
+    out = torch.empty((500, 3072, 256), dtype=torch.uint8, device="cuda")
+    seen = torch.empty((corr.PKT_SLOTS,), dtype=torch.uint8, device="cuda")
+    cnt = torch.empty((corr.PKT_COUNTERS,), dtype=torch.int32, device="cuda")
+    corr.ingest_packets(p, 9, out=out, seen=seen, counters=cnt)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        corr.ingest_packets(p, 9, out=out, seen=seen, counters=cnt, stream=torch.cuda.current_stream())
+    for first in (0, 5000, 60000):
+        sel = lane[first:first + 4003]
+        p.copy_(torch.from_numpy(np.ascontiguousarray(sel)))
+        g.replay()
+        torch.cuda.synchronize()
+        want_v, want_c = oracle.ingest(sel, 9)
+        assert np.array_equal(cnt.cpu().numpy().astype(np.int64), want_c)
+        assert np.array_equal(out.cpu().numpy(), want_v)

@@ -117,3 +117,32 @@ def _check_all_calls(N, F, T, zero_invalid):
     assert np.array_equal(tri.cpu().numpy(), oracle.to_int32(vis))
     assert np.array_equal(acc.cpu().numpy(), oracle.to_int32(2 * vis))
     assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
+
+
+def test_overlapping_launches_under_capture():
+    """A batch whose arrays take the pair, off-block and single-tile launches, which overlap
+    (two kinds of each: with invalid samples zeroed and not), replayed from a graph."""
+    shapes = [(384, 40, 300, False), (128, 200, 100, True), (250, 30, 257, False), (640, 12, 128, True)]
+    if not path_available("tc_fp8", 640):
+        pytest.skip("tc_fp8 unsupported")
+    rng = np.random.default_rng(17)
+    make = lambda: [rng.integers(0, 256, (t, f, n), dtype=np.uint8) for n, f, t, _ in shapes]
+    b = corr.Batch([dict(n_inputs=n, n_chan=f, n_time_per_int=t, path="tc_fp8", zero_invalid=z)
+                    for n, f, t, z in shapes])
+    volts = make()
+    dev = [torch.from_numpy(v).cuda() for v in volts]
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph, outs = b.capture(dev, stream=stream)
+    for _ in range(3):
+        for d, v in zip(dev, volts):
+            d.copy_(torch.from_numpy(v))
+        torch.cuda.synchronize()
+        graph.launch(stream)
+        graph.launch(stream)
+        stream.synchronize()
+        for (n, f, t, z), v, o in zip(shapes, volts, outs):
+            assert np.array_equal(o.cpu().numpy(), oracle.to_int32(oracle.xmac(v, z))), n
+        volts = make()
+    b.sync(stream)
+    graph.close()
