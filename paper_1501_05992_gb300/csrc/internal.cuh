@@ -92,6 +92,7 @@ bool tc_supported(int n_inputs, int device);
 struct TcOptions {
     long long wait_limit = 0;   // bounded-wait limit in clock64 cycles (0: about 1 s)
     bool inject_stall = false;  // test hook: make the launch's first wait expire
+    bool add_after = false;     // (set by launch_xeng_tc_batch itself)
 };
 struct TcArray {
     const uint8_t *volt;   // [nt][n_chan][ld] packed voltages (n used of each row of ld bytes)
@@ -103,6 +104,9 @@ struct TcArray {
     // beam_avg][n_chan] (zeroed by the caller); NULL for none
     int32_t *beam = nullptr;
     int beam_avg = 1, beam_t0 = 0;
+    // the channels are f0 .. f0 + n_chan - 1 of n_chan_all (0: all there are); volt, acc and
+    // beam point at the first of them
+    int f0 = 0, n_chan_all = 0;
 };
 // Whether the tensor-core path takes an array of n inputs with its rows on any byte
 // boundary (up to 256 inputs; the others come through TMA).

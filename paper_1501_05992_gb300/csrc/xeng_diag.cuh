@@ -147,6 +147,7 @@ struct ArrayParams {
     int n, n_chan, n_blocks, nt, n_stages, item_begin;
     int32_t *beam;
     int beam_ld, beam_avg, beam_t0;
+    int f0, n_chan_all;       // the channels are f0 .. of n_chan_all
 };
 
 struct Params {
@@ -156,6 +157,7 @@ struct Params {
     long long wait_limit;
     int inject_stall;
     uint32_t one, minus_one, fifteen, sixteen;   // multipliers of imad()
+    int add_after;            // the launch before zeroes what this one adds to
 };
 
 struct Item {
@@ -380,9 +382,9 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
                         const int xs = int(reinterpret_cast<uintptr_t>(x_ptr) & 3);
                         x_ptr -= xs;
                         x_rows = lane < 4 * kUnits && xs && A.n - tile - kTile + xs > 0 ? A.nt - xt : 0;
-                        edge = it.f == 0 || it.f == A.n_chan - 1;
+                        edge = it.f + A.f0 == 0 || it.f + A.f0 == A.n_chan_all - 1;
                         lo = A.volt;
-                        hi = A.volt + (long long)A.nt * row_t;
+                        hi = A.volt + (A.nt - 1) * row_t + (long long)A.n_chan * A.ld;
                     }
                     // rows of this thread with a sample (none for a chunk past the inputs)
                     rows = left + sh > 0 ? A.nt - q - s * kTc : 0;
@@ -550,6 +552,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
                        peer_full = kPair ? map_rank(bar_in_full, uint32_t(rank ^ 1)) : 0u;
         int local = 0, votes = 0;
         bool ok = true;
+        if (!kFresh && p.add_after) wait_for_launch_before();
         // the epilogue warps decide together whether to go on, so that none of them is
         // ever left waiting at a named barrier (two sets of votes in turn, so that a
         // vote is not overwritten before every warp has read it)
@@ -738,7 +741,9 @@ inline cudaError_t make_params(const TcArray *arrays, int count, bool pair, Devi
         ArrayParams &P = prm.a[k];
         P.volt = A.volt;
         P.ld = A.ld ? A.ld : A.n;
-        P.row_t = (long long)P.ld * A.n_chan;
+        P.f0 = A.f0;
+        P.n_chan_all = A.n_chan_all ? A.n_chan_all : A.n_chan;
+        P.row_t = (long long)P.ld * P.n_chan_all;
         P.acc = A.acc;
         P.n = A.n;
         P.n_chan = A.n_chan;
@@ -748,7 +753,7 @@ inline cudaError_t make_params(const TcArray *arrays, int count, bool pair, Devi
         P.n_stages = (A.nt + kTc - 1) / kTc;
         P.item_begin = int(items);
         P.beam = A.beam;
-        P.beam_ld = A.n_chan;
+        P.beam_ld = P.n_chan_all;
         P.beam_avg = A.beam_avg > 0 ? A.beam_avg : 1;
         P.beam_t0 = A.beam_t0;
         items += (long long)A.n_chan * P.n_blocks;
@@ -759,6 +764,7 @@ inline cudaError_t make_params(const TcArray *arrays, int count, bool pair, Devi
     prm.status = status;
     prm.wait_limit = opt.wait_limit > 0 ? opt.wait_limit : kDefaultWaitLimit;
     prm.inject_stall = opt.inject_stall ? 1 : 0;
+    prm.add_after = opt.add_after ? 1 : 0;
     prm.one = 1u;
     prm.minus_one = ~0u;
     prm.fifteen = 15u;

@@ -61,6 +61,91 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
     return cr == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
+// The last round of the pair kernel.  The channels of an array of one block each go round
+// the pairs of CTAs, and the last round may be nearly empty: 128 channels on 76 pairs take
+// as long as 152, 768 as long as 836.  The channels left for it can be split into up to four
+// slices of samples, which add into a zeroed triangle; the slices' items share that round.
+// Returns the slices (1: as it is) and the channels before them.  In units of 64 samples
+// per channel, 0.42 us: a slice has 16 at least (about what its stores take), and splitting
+// costs the zeroing, the adds and a launch, more where it is a second launch (about 14 and
+// 26).  256 inputs x 5000 samples: 4 channels 39.7 -> 21.3 us, 80 channels 72 -> 60 us,
+// 768 channels 359 -> 345 us (with the beam 393 -> 375); 40 channels x 20000 samples 125 ->
+// 94 us; 16 x 2200 24.9 -> 20.9 us.
+constexpr int kSplitCost = 26, kSplitCostAlone = 14;
+
+int last_round_slices(int n_chan, int nt, int pairs, int *before)
+{
+    const int stages = (nt + 63) / 64, rest = n_chan % pairs;
+    *before = n_chan - rest;
+    int best = 1, best_cost = stages - (*before ? kSplitCost : kSplitCostAlone);
+    for (int s = 2; s <= kTcMaxArrays && stages >= 16 * s && rest > 0; ++s) {
+        const int cost = (rest * s + pairs - 1) / pairs * ((stages + s - 1) / s);
+        if (cost < best_cost) {
+            best = s;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+__global__ void __launch_bounds__(256) zero_kernel(int2 *__restrict__ out, size_t n)
+{
+    let_next_launch_start();
+    for (size_t e = blockIdx.x * size_t(256) + threadIdx.x; e < n; e += gridDim.x * size_t(256))
+        out[e] = make_int2(0, 0);
+    wait_for_launch_before();
+}
+
+cudaError_t launch_pairs(const TcArray *arrays, int count, bool alone, bool fresh, bool zero_invalid, int dev,
+                         DeviceStatus *status, const TcOptions &opt, cudaStream_t s, int *launches)
+{
+    int sms = 0;
+    cudaError_t e = alone ? cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) : cudaSuccess;
+    if (e != cudaSuccess) return e;
+    const TcArray &A = arrays[0];
+    int before = 0;
+    const int slices = alone && sms > 1 ? last_round_slices(A.n_chan, A.nt, sms / 2, &before) : 1;
+    if (slices == 1) {
+        e = launch_xeng_pair(arrays, count, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+        *launches += e == cudaSuccess;
+        return e;
+    }
+    TcArray part[kTcMaxArrays];
+    const int rest = A.n_chan - before, step = ((A.nt + 63) / 64 + slices - 1) / slices * 64;
+    const size_t triangle = size_t(n_pairs(A.n));
+    for (int k = 0; k < slices; ++k) {
+        TcArray &p = part[k] = A;
+        const long long ld = A.ld ? A.ld : A.n;
+        p.f0 = before;
+        p.n_chan = rest;
+        p.n_chan_all = A.n_chan;
+        p.nt = k + 1 < slices ? step : A.nt - k * step;
+        p.volt = A.volt + before * ld + k * step * (ld * A.n_chan);
+        p.acc = A.acc + size_t(before) * triangle * 2;
+        p.beam_t0 = A.beam_t0 + k * step;
+        if (A.beam) p.beam = A.beam + before;
+    }
+    if (fresh) {
+        e = launch_overlapping(zero_kernel, sms, 256, 0, *launches > 0, s, reinterpret_cast<int2 *>(part[0].acc),
+                               triangle * rest);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    if (before) {
+        TcArray head = A;
+        head.n_chan = before;
+        head.n_chan_all = A.n_chan;
+        e = launch_xeng_pair(&head, 1, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    TcOptions last = opt;
+    last.add_after = fresh;
+    e = launch_xeng_pair(part, slices, false, zero_invalid, dev, status, last, *launches > 0, s);
+    *launches += e == cudaSuccess;
+    return e;
+}
+
 // The launches of the arrays of one mode, longest integrations first (a CTA's
 // last items are then its shortest).
 // The launches of one call write disjoint parts of the output and may overlap: each lets
@@ -81,9 +166,10 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     int n = 0;
     for (int k = 0; k < m; ++k)
         if (sorted[k].n > kTile) part[n++] = sorted[k];
-    if (n) e = launch_xeng_pair(part, n, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+    // other launches of the call would fill the last round
+    const bool alone = count == 1 && n == 1 && part[0].n <= 2 * kTile;
+    if (n) e = launch_pairs(part, n, alone, fresh, zero_invalid, dev, status, opt, s, launches);
     if (e != cudaSuccess) return e;
-    *launches += n > 0;
     n = 0;
     CUtensorMap maps[kTcMaxArrays];
     for (int k = 0; k < m; ++k) {

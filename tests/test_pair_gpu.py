@@ -119,6 +119,15 @@ def _check_all_calls(N, F, T, zero_invalid):
     assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
 
 
+# long integrations whose last round of channels is split into slices of samples: fewer
+# channels than CTA pairs, a few more, on and off 16-byte rows, a last slice of one sample
+@pytest.mark.parametrize("N,F,T", [(256, 1, 2048), (256, 3, 4097), (250, 5, 3073), (131, 38, 2111), (255, 77, 1999),
+                                   (256, 79, 5000), (250, 80, 4990), (192, 155, 1057)])
+@pytest.mark.parametrize("zero_invalid", [False, True])
+def test_last_round_in_slices(N, F, T, zero_invalid):
+    _check_all_calls(N, F, T, zero_invalid)
+
+
 def test_overlapping_launches_under_capture():
     """A batch whose arrays take the pair, off-block and single-tile launches, which overlap
     (two kinds of each: with invalid samples zeroed and not), replayed from a graph."""
