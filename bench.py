@@ -308,7 +308,7 @@ def load_peaks():
 
 
 def measured_traffic(kernel_src: str, profile_md: str, workload: str):
-    """DRAM bytes per launch from the committed ncu summary, but only while the
+    """DRAM bytes per integration from the committed ncu summary, but only while the
     kernel source still matches the one the counters were taken from."""
     import hashlib
     import re
@@ -318,7 +318,7 @@ def measured_traffic(kernel_src: str, profile_md: str, workload: str):
     except OSError:
         return None
     m = re.search(r"sha256 prefix `([0-9a-f]{16})`", text)
-    t = re.search(r"traffic_bytes_per_full_band_launch: ([0-9.e+]+)", text)
+    t = re.search(r"traffic_bytes_per_full_band_integration: ([0-9.e+]+)", text)
     if not m or not t or m.group(1) != sha or workload != "full_band":
         return None
     return float(t.group(1))
@@ -830,9 +830,10 @@ def run_ours(args, world, rank, local):
     avg_ms = xe_ms / max(1, xe_timed)
     main_path = paths[max(range(len(arrays)), key=lambda a: arrays[a][0] ** 2 * arrays[a][1] * arrays[a][2])]
     roof = roofline_for(main_path, ops_per_launch, avg_ms, peaks, src, sm_count, measured_probes(dev))
-    roof["traffic"] = (measured_traffic(os.path.join(ROOT, "paper_1501_05992_gb300", "csrc", "xeng_diag.cuh"),
-                                        os.path.join(ROOT, "profiles", "xeng_pair_full_band_traffic.md"),
-                                        args.workload) if main_path == "tc_fp8" else None)
+    traffic = (measured_traffic(os.path.join(ROOT, "paper_1501_05992_gb300", "csrc", "xeng_diag.cuh"),
+                                os.path.join(ROOT, "profiles", "xeng_pair_full_band_traffic.md"),
+                                args.workload) if main_path == "tc_fp8" else None)
+    roof["traffic"] = traffic * n_int / max(1, xe_per_step) if traffic else None    # per launch
     roof["kernel"] = {"cudacore": "xeng_dp4a_kernel", "mma_i8": "xeng_mma8_kernel",
                       "tc_fp8": "xeng_pair_kernel"}[main_path]
     roof["launches_per_step"] = xe_per_step
