@@ -61,8 +61,8 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
     return cr == CUDA_SUCCESS ? cudaSuccess : cudaErrorInvalidValue;
 }
 
-// The last round of the pair kernel.  The channels of an array of one block each go round
-// the pairs of CTAs, and the last round may be nearly empty: 128 channels on 76 pairs take
+// The last round of an array of one block (or one tile) per channel.  Its channels go round
+// the pairs of CTAs (the CTAs), and the last round may be nearly empty: 128 channels on 76 pairs take
 // as long as 152, 768 as long as 836.  The channels left for it can be split into up to four
 // slices of samples, which add into a zeroed triangle; the slices' items share that round.
 // Returns the slices (1: as it is) and the channels before them.  In units of 64 samples
@@ -70,16 +70,17 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
 // costs the zeroing, the adds and a launch, more where it is a second launch (about 14 and
 // 26).  256 inputs x 5000 samples: 4 channels 39.7 -> 21.3 us, 80 channels 72 -> 60 us,
 // 768 channels 359 -> 345 us (with the beam 393 -> 375); 40 channels x 20000 samples 125 ->
-// 94 us; 16 x 2200 24.9 -> 20.9 us.
+// 94 us; 16 x 2200 24.9 -> 20.9 us.  128 inputs x 5000 samples: 40 channels 37.5 -> 20.9 us,
+// 160 channels 68 -> 52 us, 768 channels 188 -> 171 us.
 constexpr int kSplitCost = 26, kSplitCostAlone = 14;
 
-int last_round_slices(int n_chan, int nt, int pairs, int *before)
+int last_round_slices(int n_chan, int nt, int workers, int *before)
 {
-    const int stages = (nt + 63) / 64, rest = n_chan % pairs;
+    const int stages = (nt + 63) / 64, rest = n_chan % workers;
     *before = n_chan - rest;
     int best = 1, best_cost = stages - (*before ? kSplitCost : kSplitCostAlone);
     for (int s = 2; s <= kTcMaxArrays && stages >= 16 * s && rest > 0; ++s) {
-        const int cost = (rest * s + pairs - 1) / pairs * ((stages + s - 1) / s);
+        const int cost = (rest * s + workers - 1) / workers * ((stages + s - 1) / s);
         if (cost < best_cost) {
             best = s;
             best_cost = cost;
@@ -96,17 +97,20 @@ __global__ void __launch_bounds__(256) zero_kernel(int2 *__restrict__ out, size_
     wait_for_launch_before();
 }
 
-cudaError_t launch_pairs(const TcArray *arrays, int count, bool alone, bool fresh, bool zero_invalid, int dev,
-                         DeviceStatus *status, const TcOptions &opt, cudaStream_t s, int *launches)
+// The pair kernel's (pair) or the tile kernel's launches of these arrays.  alone: they are one
+// array, whose channels are all that the call computes.
+cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alone, bool fresh, bool zero_invalid,
+                          int dev, DeviceStatus *status, const TcOptions &opt, cudaStream_t s, int *launches)
 {
+    const auto launch = pair ? launch_xeng_pair : launch_xeng_tile;
     int sms = 0;
     cudaError_t e = alone ? cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) : cudaSuccess;
     if (e != cudaSuccess) return e;
     const TcArray &A = arrays[0];
     int before = 0;
-    const int slices = alone && sms > 1 ? last_round_slices(A.n_chan, A.nt, sms / 2, &before) : 1;
+    const int slices = alone && sms > 1 ? last_round_slices(A.n_chan, A.nt, pair ? sms / 2 : sms, &before) : 1;
     if (slices == 1) {
-        e = launch_xeng_pair(arrays, count, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+        e = launch(arrays, count, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
         *launches += e == cudaSuccess;
         return e;
     }
@@ -135,13 +139,13 @@ cudaError_t launch_pairs(const TcArray *arrays, int count, bool alone, bool fres
         TcArray head = A;
         head.n_chan = before;
         head.n_chan_all = A.n_chan;
-        e = launch_xeng_pair(&head, 1, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+        e = launch(&head, 1, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
         if (e != cudaSuccess) return e;
         ++*launches;
     }
     TcOptions last = opt;
     last.add_after = fresh;
-    e = launch_xeng_pair(part, slices, false, zero_invalid, dev, status, last, *launches > 0, s);
+    e = launch(part, slices, false, zero_invalid, dev, status, last, *launches > 0, s);
     *launches += e == cudaSuccess;
     return e;
 }
@@ -168,7 +172,7 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
         if (sorted[k].n > kTile) part[n++] = sorted[k];
     // other launches of the call would fill the last round
     const bool alone = count == 1 && n == 1 && part[0].n <= 2 * kTile;
-    if (n) e = launch_pairs(part, n, alone, fresh, zero_invalid, dev, status, opt, s, launches);
+    if (n) e = launch_blocks(true, part, n, alone, fresh, zero_invalid, dev, status, opt, s, launches);
     if (e != cudaSuccess) return e;
     n = 0;
     CUtensorMap maps[kTcMaxArrays];
@@ -184,8 +188,8 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     n = 0;
     for (int k = 0; k < m; ++k)
         if ((sorted[k].n + kTile - 1) / kTile % 2) part[n++] = sorted[k];
-    if (n) e = launch_xeng_tile(part, n, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
-    *launches += n > 0;
+    if (n) e = launch_blocks(false, part, n, count == 1 && part[0].n <= kTile, fresh, zero_invalid, dev, status, opt, s,
+                             launches);
     return e;
 }
 

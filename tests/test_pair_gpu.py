@@ -122,7 +122,8 @@ def _check_all_calls(N, F, T, zero_invalid):
 # long integrations whose last round of channels is split into slices of samples: fewer
 # channels than CTA pairs, a few more, on and off 16-byte rows, a last slice of one sample
 @pytest.mark.parametrize("N,F,T", [(256, 1, 2048), (256, 3, 4097), (250, 5, 3073), (131, 38, 2111), (255, 77, 1999),
-                                   (256, 79, 5000), (250, 80, 4990), (192, 155, 1057)])
+                                   (256, 79, 5000), (250, 80, 4990), (192, 155, 1057), (128, 3, 4097), (100, 155, 2111),
+                                   (65, 160, 1999)])
 @pytest.mark.parametrize("zero_invalid", [False, True])
 def test_last_round_in_slices(N, F, T, zero_invalid):
     _check_all_calls(N, F, T, zero_invalid)
