@@ -131,17 +131,6 @@ __device__ __forceinline__ void tma_load_3d(uint32_t dst, const CUtensorMap *map
         : "memory");
 }
 
-// The same into this offset of every CTA of `mask`, counted on each one's barrier.
-__device__ __forceinline__ void tma_load_3d_multicast(uint32_t dst, const CUtensorMap *map, uint32_t bar, int x, int y,
-                                                      int z, uint16_t mask)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.multicast::cluster"
-        " [%0], [%1, {%2, %3, %4}], [%5], %6;" ::"r"(dst),
-        "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(bar), "h"(mask)
-        : "memory");
-}
-
 __device__ __forceinline__ uint64_t smem_desc(uint32_t saddr, uint32_t lbo, uint32_t sbo)
 {
     uint64_t d = 0;
@@ -383,7 +372,7 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool fresh, bool 
 cudaError_t launch_xeng_tile(const TcArray *arrays, int count, bool fresh, bool zero_invalid, int dev,
                              DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
 // The rest of their triangles (xeng_off.cu), for arrays of 257 or more inputs;
-// maps[k] is array k's tensor map (boxes of 128 inputs x 1 channel x 32 samples).
+// maps[k] is array k's tensor map (boxes of 128 inputs x 1 channel x 64 samples).
 cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int count, bool fresh, bool zero_invalid,
                             int dev, DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
 

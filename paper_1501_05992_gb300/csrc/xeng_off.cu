@@ -19,19 +19,19 @@
 // warps 8-23 converters (two teams of eight that take alternate 64-sample stages;
 // in a team, half of the threads convert I and half J), warp 24 TMEM allocation and
 // (leader CTA) the MMA issuer, warp 25 the TMA producer (one thread; a ring of
-// six 16 KB stages).  The TMA unit takes between four and five cycles per 128-byte
-// row, i.e. 0.3 us for a stage's two tiles, so each CTA loads half of I's samples and
-// multicasts them to both (1024 inputs x 128 channels x 10000 samples, both kernels:
-// 1.87 -> 1.80 ms with the cheaper decoding), and nothing is prefetched into L2 (a
-// prefetch takes the same time).  TMEM holds two accumulators.
+// six 16 KB stages).  Each CTA loads both of its tiles, I as well as its own half of J:
+// the TMA unit takes between four and five cycles per 128-byte row, i.e. 0.3 us for a
+// stage's two tiles, which hides behind the converters; a box holds a whole stage of a
+// tile, so a stage is two instructions.  Nothing is prefetched into L2 (a prefetch
+// takes the same time).  TMEM holds two accumulators.
 //
 // What bounds it: a stage takes 0.43 us, 0.24 us of it the tensor pipe; the converters'
 // turn-around (waits, decoding, stores, proxy fence) is the rest, and without their
 // decoding a stage takes 0.36 us.  Against one 128-input tile per CTA with its
 // neighbour's (the form before), together with xeng_pair.cu's and xeng_tile.cu's
-// share: 1024 inputs x 128 channels x 10000 samples 2.04 -> 1.74 ms, 512 x 384 x 5000
-// 0.80 -> 0.71 ms, 384 x 384 x 5000 0.49 -> 0.45 ms, 500 samples added to 512 x 768 0.49
-// -> 0.41 ms.
+// share: 1024 inputs x 128 channels x 10000 samples 2.04 -> 1.73 ms, 512 x 384 x 5000
+// 0.80 -> 0.70 ms, 384 x 384 x 5000 0.49 -> 0.45 ms, 500 samples added to 512 x 768 0.49
+// -> 0.42 ms.
 #include <cuda.h>
 #include <cudaTypedefs.h>
 
@@ -156,7 +156,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
     if (threadIdx.x == 0) {
         for (int s = 0; s < kPackedStages; ++s) {
             mbar_init(bar_packed_full(s), 1);
-            mbar_init(bar_packed_empty(s), 2 * kTeamWarps);
+            mbar_init(bar_packed_empty(s), kTeamWarps);
         }
         for (int s = 0; s < kPlaneStages; ++s) {
             mbar_init(bar_plane_full(s), 2 * kTeamWarps);
@@ -206,11 +206,8 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
                     }
                     const uint32_t full = bar_packed_full(stage), dst = sbase + kSmPacked + stage * kPackedBytes;
                     mbar_expect_tx(full, kPackedBytes);
-                    // this CTA's half of I's samples into both CTAs, then its own J tile
-                    tma_load_3d_multicast(dst + rank * kPlaneBytes / 2, tmap, full, xi, it.f, s * kTc + rank * kTc / 2,
-                                          uint16_t(3));
+                    tma_load_3d(dst, tmap, full, xi, it.f, s * kTc);
                     tma_load_3d(dst + kPlaneBytes, tmap, full, xj, it.f, s * kTc);
-                    tma_load_3d(dst + kPlaneBytes + kPlaneBytes / 2, tmap, full, xj, it.f, s * kTc + kTc / 2);
                     issued |= 1u << stage;
                     issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
                     if (++stage == kPackedStages) {
@@ -219,9 +216,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
                     }
                 }
             }
-            // every issued load must have landed before the CTA may exit (after a timeout
-            // also those of I that the pair does not wait for)
-            if (!ok) __nanosleep(100000);
+            // every issued load must have landed before the CTA may exit
             for (int k = 0; k < kPackedStages; ++k) {
                 if (!((issued >> k) & 1u)) continue;
                 const long long t0 = clock64();
@@ -338,9 +333,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
                 __syncwarp();
                 if (lane == 0) {
                     remote_arrive(map_rank(bar_plane_full(cstage), 0));
-                    // the slot takes loads of both CTAs (I), so both producers wait for both
                     mbar_arrive(bar_packed_empty(pstage));
-                    remote_arrive(map_rank(bar_packed_empty(pstage), uint32_t(rank ^ 1)));
                 }
                 pstage += kTeams;
                 if (pstage >= kPackedStages) {

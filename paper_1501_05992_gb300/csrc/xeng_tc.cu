@@ -24,7 +24,7 @@ namespace corr {
 namespace {
 
 constexpr int kTile = 128;
-constexpr int kBoxSamples = 32;               // samples of a tensor-map box (half a stage)
+constexpr int kBoxSamples = 64;               // samples of a tensor-map box (a stage)
 constexpr size_t kSmemNeeded = 227 * 1024;    // the largest kernel's shared memory, at most
 
 PFN_cuTensorMapEncodeTiled_v12000 g_encode = nullptr;
