@@ -111,6 +111,14 @@ struct TcArray {
 // Whether the tensor-core path takes an array of n inputs with its rows on any byte
 // boundary (up to 256 inputs; the others come through TMA).
 bool tc_any_rows(int n);
+// Whether a 32-bit word on a word boundary that holds a byte of channel f's row of n bytes
+// can reach over an end of the array (of n_chan such rows per sample).  Such a word holds up
+// to three bytes of its neighbours, so with rows of one or two bytes it is not the first and
+// the last channel alone.
+__host__ __device__ inline bool words_reach_over(int f, int n_chan, int n)
+{
+    return (long long)f * n < 3 || (long long)(n_chan - 1 - f) * n < 3;
+}
 // Samples per padded copy for the tensor-core path when n % 16 != 0: the
 // whole integration if it fits kTcPadCap bytes, else chunks of a multiple
 // of 64 samples.

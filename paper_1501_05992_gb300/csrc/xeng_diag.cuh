@@ -358,7 +358,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
         // rows on any byte: this thread's inputs from its chunk on, its rows' offset from
         // a word boundary, whether the item has such offsets; the extra word's address and
         // the number of samples it is there for; the array's bytes and whether the item
-        // has words that reach over their ends (its first and last channels)
+        // has words that reach over their ends
         int left = kTile, sh = 0, x_rows = 0;
         bool skew = false, edge = false;
         const uint8_t *x_ptr = nullptr, *lo = nullptr, *hi = nullptr;
@@ -382,7 +382,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
                         const int xs = int(reinterpret_cast<uintptr_t>(x_ptr) & 3);
                         x_ptr -= xs;
                         x_rows = lane < 4 * kUnits && xs && A.n - tile - kTile + xs > 0 ? A.nt - xt : 0;
-                        edge = it.f + A.f0 == 0 || it.f + A.f0 == A.n_chan_all - 1;
+                        edge = words_reach_over(it.f + A.f0, A.n_chan_all, A.n);
                         lo = A.volt;
                         hi = A.volt + (A.nt - 1) * row_t + (long long)A.n_chan * A.ld;
                     }
