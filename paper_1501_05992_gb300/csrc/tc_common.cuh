@@ -81,6 +81,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// Limit of the waits for copies and MMAs in flight before their memory is given up (a
+// parameter of the launches, Params::drain_limit).  They end whatever the roles' waits came
+// to, so these waits don't take the caller's limit, which may be shorter than they need.
+constexpr long long kDefaultWaitLimit = 1LL << 31;
+
 // Warp-wide bounded wait: lane 0 polls (with an optional back-off), then every
 // lane confirms once, so each lane gets the barrier's acquire ordering while
 // only one lane keeps hitting shared memory.
@@ -270,6 +275,11 @@ __device__ __forceinline__ void store_async4(uint32_t addr, const uint32_t *v, u
                      addr),
                  "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3]), "r"(bar)
                  : "memory");
+}
+
+__device__ __forceinline__ void store_peer(uint32_t addr, int v)
+{
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
 }
 
 __device__ __forceinline__ bool mbar_try_cluster(uint32_t bar, uint32_t parity)

@@ -116,7 +116,6 @@ __device__ __forceinline__ uint32_t idesc_tile(int inputs)
     const uint32_t n = inputs >= 128 ? 128u : uint32_t((inputs + 15) & ~15);
     return (1u << 4) | (1u << 15) | (1u << 16) | ((n >> 3) << 17) | ((128u >> 4) << 24);
 }
-constexpr long long kDefaultWaitLimit = 1LL << 31;
 
 // shared-memory map (offsets from the 1024-aligned base, the same in both CTAs)
 constexpr int kSmPlanes = 0;
@@ -158,6 +157,7 @@ struct Params {
     int inject_stall;
     uint32_t one, minus_one, fifteen, sixteen;   // multipliers of imad()
     int add_after;            // the launch before zeroes what this one adds to
+    long long drain_limit;
 };
 
 struct Item {
@@ -237,6 +237,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + kSmMisc);
     volatile int *abort = reinterpret_cast<volatile int *>(smem + kSmMisc + 8);
     volatile int *epi_ok = reinterpret_cast<volatile int *>(smem + kSmMisc + 16);
+    volatile int *sent = reinterpret_cast<volatile int *>(smem + kSmMisc + 96);   // items sent: to this CTA, by it
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < kPlaneStages; ++s) {
@@ -329,7 +330,7 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
             }
             __syncwarp();
             const long long t0 = clock64();
-            while (!mbar_try(bar_drain, 0) && clock64() - t0 < p.wait_limit) {
+            while (!mbar_try(bar_drain, 0) && clock64() - t0 < p.drain_limit) {
             }
         }
     } else if (warp >= kFirstConvWarp) {
@@ -713,8 +714,11 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
             // the next item's vote follows every read of the buffers; a failed wait shows in it
             if (!ok && item + item_step < p.n_items) agree(false);
         }
-        // after a timeout, rows may still be on their way to the pair's inbox
-        if (kPair && !ok) __nanosleep(100000);
+        // all rows of an item are sent, or none, so the pair knows what to expect
+        if (kPair && threadIdx.x == 0) {
+            sent[1] = local;
+            store_peer(map_rank(sbase + kSmMisc + 96, uint32_t(rank ^ 1)), local);
+        }
     }
 
     __syncwarp();
@@ -725,6 +729,15 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
     fence_after();
     if (warp == kMmaWarp) {
         tmem_dealloc<kPair>(tmem, kTmemCols);
+    }
+    if (kPair && warp == kMmaWarp && lane == 0 && sent[0] > 0) {
+        // after a timeout the rows of the pair's last item may still be on their way into the
+        // inbox, which may not even be armed for them: they land before this CTA leaves
+        if (sent[0] > sent[1]) mbar_expect_tx(bar_in_full, kInboxBytes);
+        const uint32_t parity = uint32_t(sent[0] - 1) & 1u;
+        const long long t0 = clock64();
+        while (!mbar_try(bar_in_full, parity) && clock64() - t0 < p.drain_limit) {
+        }
     }
     wait_for_launch_before();
 }
@@ -763,6 +776,7 @@ inline cudaError_t make_params(const TcArray *arrays, int count, bool pair, Devi
     prm.n_items = int(items);
     prm.status = status;
     prm.wait_limit = opt.wait_limit > 0 ? opt.wait_limit : kDefaultWaitLimit;
+    prm.drain_limit = kDefaultWaitLimit;
     prm.inject_stall = opt.inject_stall ? 1 : 0;
     prm.add_after = opt.add_after ? 1 : 0;
     prm.one = 1u;

@@ -56,7 +56,6 @@ static_assert(kPackedStages % kTeams == 0 && kPlaneStages >= kTeams, "slots per 
 constexpr int kFirstConvWarp = kEpiWarps, kMmaWarp = kFirstConvWarp + kConvWarps, kTmaWarp = kMmaWarp + 1;
 constexpr int kThreads = (kTmaWarp + 1) * 32;
 constexpr int kTmemCols = 512;
-constexpr long long kDefaultWaitLimit = 1LL << 31;
 
 // shared-memory map (offsets from the 1024-aligned base, the same in both CTAs)
 constexpr int kSmPlanes = 0;
@@ -81,6 +80,7 @@ struct Params {
     long long wait_limit;
     int inject_stall;
     uint32_t one, fifteen;                    // multipliers of imad()
+    long long drain_limit;
 };
 
 struct Tmaps {
@@ -220,7 +220,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
             for (int k = 0; k < kPackedStages; ++k) {
                 if (!((issued >> k) & 1u)) continue;
                 const long long t0 = clock64();
-                while (!mbar_try(bar_packed_full(k), (issued_phase >> k) & 1u) && clock64() - t0 < p.wait_limit) {
+                while (!mbar_try(bar_packed_full(k), (issued_phase >> k) & 1u) && clock64() - t0 < p.drain_limit) {
                 }
             }
         }
@@ -271,7 +271,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
             if (lane == 0) commit_own(bar_drain);
             __syncwarp();
             const long long t0 = clock64();
-            while (!mbar_try(bar_drain, 0) && clock64() - t0 < p.wait_limit) {
+            while (!mbar_try(bar_drain, 0) && clock64() - t0 < p.drain_limit) {
             }
         }
     } else if (warp >= kFirstConvWarp) {
@@ -530,6 +530,7 @@ cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int 
     prm.n_items = int(items);
     prm.status = status;
     prm.wait_limit = opt.wait_limit > 0 ? opt.wait_limit : kDefaultWaitLimit;
+    prm.drain_limit = kDefaultWaitLimit;
     prm.inject_stall = opt.inject_stall ? 1 : 0;
     prm.one = 1u;
     prm.fifteen = 15u;
