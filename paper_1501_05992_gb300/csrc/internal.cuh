@@ -107,6 +107,7 @@ struct TcArray {
     // the channels are f0 .. f0 + n_chan - 1 of n_chan_all (0: all there are); volt, acc and
     // beam point at the first of them
     int f0 = 0, n_chan_all = 0;
+    bool last_as_block = false;   // an odd number of tiles: the last is a block whose second tile is empty
 };
 // Whether the tensor-core path takes an array of n inputs with its rows on any byte
 // boundary (up to 256 inputs; the others come through TMA).

@@ -761,7 +761,7 @@ inline cudaError_t make_params(const TcArray *arrays, int count, bool pair, Devi
         P.n = A.n;
         P.n_chan = A.n_chan;
         P.first = pair ? 0 : (n_tiles - 1) * kTile;
-        P.n_blocks = pair ? n_tiles / 2 : 1;
+        P.n_blocks = pair ? (n_tiles + (A.last_as_block ? 1 : 0)) / 2 : 1;
         P.nt = A.nt;
         P.n_stages = (A.nt + kTc - 1) / kTc;
         P.item_begin = int(items);

@@ -5,7 +5,8 @@
 //   - the 256-input blocks on the diagonal (tiles 2 b, 2 b + 1): CTA pairs,
 //     xeng_pair.cu;
 //   - the last tile alone, where the number of tiles is odd (an array of up to 128
-//     inputs is nothing else): single CTAs, xeng_tile.cu;
+//     inputs is nothing else): single CTAs, xeng_tile.cu, or a block whose second tile is
+//     empty (last_tile_as_block);
 //   - the tiles off those blocks, from 257 inputs on: CTA pairs, xeng_off.cu.
 // Each is one persistent launch over every channel of up to kTcMaxArrays arrays.
 // Whether invalid samples are zeroed (CORR_ZERO_INVALID) and whether the launch stores
@@ -150,6 +151,24 @@ cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alon
     return e;
 }
 
+int tiles_of(const TcArray &A) { return (A.n + kTile - 1) / kTile; }
+
+// Whether the last tile of an array with an odd number of tiles, more than two, goes to the
+// pair kernel as a block whose second tile is empty: where the pairs of CTAs that its items
+// take are idle in the last round of the others, of two at most.  It saves the third launch
+// of a call (2 us of the host's time, and its start) and costs nothing then: 384 inputs x 20
+// channels x 100 samples 14.2 -> 12.4 us, 384 x 40 x 1000 32.8 -> 30.8, 640 x 20 x 100 22.6 ->
+// 20.6, 896 x 9 x 200 24.5 -> 22.6.  With a round more it is slower (384 x 26 x 1000 18.8 ->
+// 28.9 us), and with three rounds on short integrations (640 x 28 x 100 24.7 -> 26.7).
+bool last_tile_as_block(const TcArray &A, int sms)
+{
+    const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2;
+    if (tiles % 2 == 0 || tiles == 1 || pairs < 1) return false;
+    const long long others = (long long)A.n_chan * (half + half * half);     // blocks, and the tiles off them
+    const long long rounds = (others + pairs - 1) / pairs;
+    return rounds <= 2 && others + A.n_chan <= rounds * pairs;
+}
+
 // The launches of the arrays of one mode, longest integrations first (a CTA's
 // last items are then its shortest).
 // The launches of one call write disjoint parts of the output and may overlap: each lets
@@ -167,6 +186,12 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     for (int x = 1; x < m; ++x)
         for (int y = x; y > 0 && sorted[y].nt > sorted[y - 1].nt; --y) std::swap(sorted[y], sorted[y - 1]);
     cudaError_t e = cudaSuccess;
+    if (count == 1 && m == 1) {
+        int sms = 0;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        sorted[0].last_as_block = last_tile_as_block(sorted[0], sms);
+    }
     int n = 0;
     for (int k = 0; k < m; ++k)
         if (sorted[k].n > kTile) part[n++] = sorted[k];
@@ -187,7 +212,7 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     *launches += n > 0;
     n = 0;
     for (int k = 0; k < m; ++k)
-        if ((sorted[k].n + kTile - 1) / kTile % 2) part[n++] = sorted[k];
+        if (tiles_of(sorted[k]) % 2 && !sorted[k].last_as_block) part[n++] = sorted[k];
     if (n) e = launch_blocks(false, part, n, count == 1 && part[0].n <= kTile, fresh, zero_invalid, dev, status, opt, s,
                              launches);
     return e;

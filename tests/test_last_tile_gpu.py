@@ -1,0 +1,35 @@
+"""The last of an odd number of tiles, alone or as a block with an empty second tile: channel
+counts on both sides of the rule that chooses, one input to a whole tile in it, stored, added
+and with the fused beam, bit-exact against the oracle."""
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1501_05992_gb300 import corr
+
+from _gpu import path_available
+
+pytestmark = pytest.mark.gpu
+
+
+# on 76 pairs of CTAs: one round of pairs, two rounds, a round more with the last tile, three rounds
+@pytest.mark.parametrize("N,F,T", [(257, 25, 70), (272, 45, 65), (384, 50, 64), (640, 21, 130), (897, 5, 63),
+                                   (257, 26, 70), (304, 51, 65), (384, 38, 64), (513, 11, 130), (640, 28, 63)])
+@pytest.mark.parametrize("zero_invalid", [False, True])
+def test_last_tile_exact(N, F, T, zero_invalid):
+    if not path_available("tc_fp8", N):
+        pytest.skip("tc_fp8 unsupported")
+    volt = np.random.default_rng(N + F + T).integers(0, 256, (T, F, N), dtype=np.uint8)
+    c = corr.Correlator(N, F, 2 * T, path="tc_fp8", zero_invalid=zero_invalid)
+    d = torch.from_numpy(volt).cuda()
+    tri, beam = c.integrate_beam(d, 1)
+    c.accumulate(d)
+    c.accumulate(d)
+    acc = c.dump()
+    c.sync()
+    c.close()
+    vis = oracle.xmac(volt, zero_invalid)
+    assert np.array_equal(tri.cpu().numpy(), oracle.to_int32(vis))
+    assert np.array_equal(acc.cpu().numpy(), oracle.to_int32(2 * vis))
+    assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
