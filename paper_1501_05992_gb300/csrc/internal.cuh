@@ -20,6 +20,7 @@ constexpr int kHostChunk = 500;        // samples per host->device transfer chun
 constexpr int kHostBuffers = 3;        // device staging buffers of the host chunks
 constexpr int kTcMaxSamples = 32768;   // tcgen05 path: samples per launch (FP32 sums < 2^24)
 constexpr int kTcMaxArrays = 4;        // tcgen05 path: arrays correlated by one launch
+constexpr int kTcMaxOffParts = 8;      // and parts of an array that the kernel of the tiles off the blocks takes
 constexpr size_t kAlign = 256;
 
 __host__ __device__ inline long long n_pairs(long long n) { return n * (n + 1) / 2; }

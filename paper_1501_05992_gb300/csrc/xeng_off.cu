@@ -74,17 +74,18 @@ struct ArrayParams {
 };
 
 struct Params {
-    ArrayParams a[kTcMaxArrays];
+    ArrayParams a[kTcMaxOffParts];
     int n_arrays, n_items;
     DeviceStatus *status;
     long long wait_limit;
     int inject_stall;
     uint32_t one, fifteen;                    // multipliers of imad()
     long long drain_limit;
+    int add_after;                            // a launch before zeroes what this one adds to
 };
 
 struct Tmaps {
-    CUtensorMap m[kTcMaxArrays];
+    CUtensorMap m[kTcMaxOffParts];
 };
 
 struct Item {
@@ -398,6 +399,7 @@ xeng_off_kernel(const __grid_constant__ Tmaps tmaps, const __grid_constant__ Par
         const int il = q * 32 + lane;                // this thread's input of its J tile
         int local = 0, votes = 0;
         bool ok = true;
+        if (!kFresh && p.add_after) wait_for_launch_before();
         // the epilogue warps decide together whether to go on (two sets of votes in turn)
         auto agree = [&](bool mine) {
             volatile int *const v = epi_ok + kEpiWarps * (votes++ & 1);
@@ -493,7 +495,7 @@ int g_clusters[64] = {0};
 cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int count, bool fresh, bool zero_invalid,
                             int dev, DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s)
 {
-    if (count < 1 || count > kTcMaxArrays || dev < 0 || dev >= 64) return cudaErrorInvalidValue;
+    if (count < 1 || count > kTcMaxOffParts || dev < 0 || dev >= 64) return cudaErrorInvalidValue;
     {
         std::lock_guard<std::mutex> lock(g_mu);
         if (!g_clusters[dev]) {
@@ -531,6 +533,7 @@ cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int 
     prm.status = status;
     prm.wait_limit = opt.wait_limit > 0 ? opt.wait_limit : kDefaultWaitLimit;
     prm.drain_limit = kDefaultWaitLimit;
+    prm.add_after = opt.add_after ? 1 : 0;
     prm.inject_stall = opt.inject_stall ? 1 : 0;
     prm.one = 1u;
     prm.fifteen = 15u;

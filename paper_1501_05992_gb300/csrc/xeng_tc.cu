@@ -53,7 +53,7 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
 {
     const cuuint64_t ld = cuuint64_t(A.ld ? A.ld : A.n);
     const cuuint64_t dims[3] = {cuuint64_t(A.n), cuuint64_t(A.n_chan), cuuint64_t(A.nt)};
-    const cuuint64_t strides[2] = {ld, ld * cuuint64_t(A.n_chan)};
+    const cuuint64_t strides[2] = {ld, ld * cuuint64_t(A.n_chan_all ? A.n_chan_all : A.n_chan)};
     const cuuint32_t box[3] = {cuuint32_t(kTile), 1u, cuuint32_t(kBoxSamples)};
     const cuuint32_t estr[3] = {1u, 1u, 1u};
     const CUresult cr = encoder()(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 3, const_cast<uint8_t *>(A.volt), dims, strides,
@@ -98,6 +98,30 @@ __global__ void __launch_bounds__(256) zero_kernel(int2 *__restrict__ out, size_
     wait_for_launch_before();
 }
 
+// Channels f0 .. f0 + n_chan - 1 and samples t0 .. t0 + nt - 1 of a whole array.
+TcArray part_of(const TcArray &A, int f0, int n_chan, int t0, int nt)
+{
+    TcArray p = A;
+    const long long ld = A.ld ? A.ld : A.n;
+    p.f0 = f0;
+    p.n_chan = n_chan;
+    p.n_chan_all = A.n_chan;
+    p.nt = nt;
+    p.volt = A.volt + f0 * ld + t0 * (ld * A.n_chan);
+    p.acc = A.acc + size_t(f0) * size_t(n_pairs(A.n)) * 2;
+    p.beam_t0 = A.beam_t0 + t0;
+    if (A.beam) p.beam = A.beam + f0;
+    return p;
+}
+
+// Those channels in `slices` slices of samples, of whole stages but for the last.
+void slices_of(const TcArray &A, int f0, int n_chan, int slices, TcArray *part)
+{
+    const int step = ((A.nt + 63) / 64 + slices - 1) / slices * 64;
+    for (int k = 0; k < slices; ++k)
+        part[k] = part_of(A, f0, n_chan, k * step, k + 1 < slices ? step : A.nt - k * step);
+}
+
 // The pair kernel's (pair) or the tile kernel's launches of these arrays.  alone: they are one
 // array, whose channels are all that the call computes.
 cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alone, bool fresh, bool zero_invalid,
@@ -116,20 +140,9 @@ cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alon
         return e;
     }
     TcArray part[kTcMaxArrays];
-    const int rest = A.n_chan - before, step = ((A.nt + 63) / 64 + slices - 1) / slices * 64;
+    const int rest = A.n_chan - before;
     const size_t triangle = size_t(n_pairs(A.n));
-    for (int k = 0; k < slices; ++k) {
-        TcArray &p = part[k] = A;
-        const long long ld = A.ld ? A.ld : A.n;
-        p.f0 = before;
-        p.n_chan = rest;
-        p.n_chan_all = A.n_chan;
-        p.nt = k + 1 < slices ? step : A.nt - k * step;
-        p.volt = A.volt + before * ld + k * step * (ld * A.n_chan);
-        p.acc = A.acc + size_t(before) * triangle * 2;
-        p.beam_t0 = A.beam_t0 + k * step;
-        if (A.beam) p.beam = A.beam + before;
-    }
+    slices_of(A, before, rest, slices, part);
     if (fresh) {
         e = launch_overlapping(zero_kernel, sms, 256, 0, *launches > 0, s, reinterpret_cast<int2 *>(part[0].acc),
                                triangle * rest);
@@ -137,9 +150,7 @@ cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alon
         ++*launches;
     }
     if (before) {
-        TcArray head = A;
-        head.n_chan = before;
-        head.n_chan_all = A.n_chan;
+        const TcArray head = part_of(A, 0, before, 0, A.nt);
         e = launch(&head, 1, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
         if (e != cudaSuccess) return e;
         ++*launches;
@@ -169,6 +180,136 @@ bool last_tile_as_block(const TcArray &A, int sms)
     return rounds <= 2 && others + A.n_chan <= rounds * pairs;
 }
 
+// The last round of a call of one array of more than 256 inputs.  Its items, the blocks and the
+// tiles off them, go round the pairs of CTAs together, and the last round may be nearly empty
+// (512 inputs x 20 channels: 80 items on 76 pairs).  Then the tiles off the blocks of as many
+// channels as that round needs, and the last tiles of an odd number of them (or these alone),
+// can go in slices of samples, which add into zeroed elements.  Costs are in units of 64
+// samples per item as for last_round_slices; slices cost about 20, and one per MB that is
+// zeroed and added to: 512 inputs x 20 channels x 5000 samples 78.2 -> 57.6 us, 1024 x 5 x
+// 9500 131 -> 92, 384 x 38 x 5000 74.0 -> 59.7, 640 x 24 x 5000 111 -> 96.  More last tiles than
+// SMs stay whole (384 x 160 x 7000 286 us, 295 in slices), and so does what would save less than
+// a sixteenth: in many rounds the last one is cheap, since power bounds the others (512 x 300 x
+// 9000 927 us, 939 in slices).
+struct LargePlan {
+    int off_chans = 0;        // last channels whose tiles off the blocks go in slices
+    int off_slices = 1, tile_slices = 1;
+};
+constexpr int kLargeSplitCost = 20;
+
+int rounds_of(long long items, int workers) { return int((items + workers - 1) / workers); }
+
+LargePlan plan_large(const TcArray &A, int sms)
+{
+    LargePlan plan;
+    const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2, stages = (A.nt + 63) / 64;
+    if (pairs < 1) return plan;
+    const int per_off = tiles % 2 ? half * half : half * (half - 1);
+    const long long items = (long long)A.n_chan * (half + per_off);
+    const int lone = tiles % 2 && !last_tile_as_block(A, sms) ? A.n_chan : 0;       // last tiles alone
+    const int full = int(items / pairs), left = int(items % pairs);
+    const int whole = rounds_of(items, pairs), idle = left ? sms - 2 * left : 0;
+    // whole items; the last tiles take the SMs that the last round leaves idle first
+    long long best = (long long)whole * stages;
+    if (lone > idle) best += (long long)rounds_of(lone - idle, sms) * stages;
+    best -= best / 16;
+    const long long last_rows = A.n - 2 * kTile * half;
+    const double mb_tiles = tiles % 2 ? double(A.n_chan) * double(n_pairs(last_rows)) * 8e-6 : 0.0,
+                 mb_item = 2.0 * kTile * kTile * 8e-6;
+    auto take = [&](long long cost, int chans, int so, int st) {
+        const double mb = (st > 1 ? mb_tiles * (st + 1) : 0.0) + double(chans) * per_off * mb_item * (so + 1);
+        cost += kLargeSplitCost + (long long)mb;
+        if (cost >= best) return;
+        best = cost;
+        plan.off_chans = chans;
+        plan.off_slices = so;
+        plan.tile_slices = st;
+    };
+    const int last_tiles = tiles % 2 ? A.n_chan : 0, chans = (left + per_off - 1) / per_off;
+    for (int st = 1; st <= (last_tiles && last_tiles <= sms ? kTcMaxArrays : 1) && stages >= 16 * st; ++st) {
+        const int tile_stages = (stages + st - 1) / st;
+        // slices of the last tiles alone
+        if (st > 1 && last_tiles > idle)
+            take((long long)whole * stages + (long long)rounds_of((long long)(last_tiles - idle) * st, sms) * tile_stages,
+                 0, 1, st);
+        // slices of the last round's items and of the last tiles in a round of their own
+        if (!full || !chans || chans >= A.n_chan || (last_tiles && st == 1)) continue;
+        for (int so = 2; so <= kTcMaxOffParts && stages >= 16 * so; ++so) {
+            const int off_stages = (stages + so - 1) / so,
+                      longest = last_tiles && tile_stages > off_stages ? tile_stages : off_stages;
+            take((long long)full * stages +
+                     (long long)rounds_of(2LL * chans * per_off * so + (long long)last_tiles * st, sms) * longest,
+                 chans, so, st);
+        }
+    }
+    return plan;
+}
+
+// Zeroes what the slices of a plan add to: for the last `chans` channels the elements left of
+// each row's own 256-input block, and (tiles) every channel's last tile.  A warp per row.
+__global__ void __launch_bounds__(256) zero_large_kernel(int2 *__restrict__ out, int n, int n_chan, int chans, int tiles)
+{
+    let_next_launch_start();
+    const int base = (n - 1) / kTile * kTile, rows = n - 2 * kTile, lane = threadIdx.x & 31;
+    const long long triangle = n_pairs(n), first = chans ? 2 * kTile : base;
+    for (long long r = blockIdx.x * 8LL + (threadIdx.x >> 5); r < (long long)n_chan * rows; r += gridDim.x * 8LL) {
+        const int f = int(r / rows), i = 2 * kTile + int(r - (long long)f * rows);
+        if (i < first) continue;
+        const int own = i / (2 * kTile) * (2 * kTile);
+        const bool last = tiles && i >= base;
+        const int end = last ? i + 1 : f >= n_chan - chans ? own : 0;
+        int2 *const row = out + f * triangle + n_pairs(i);
+        for (int j = (f >= n_chan - chans ? 0 : own) + lane; j < end; j += 32) row[j] = make_int2(0, 0);
+    }
+    wait_for_launch_before();
+}
+
+// The launches of a call of one array of more than 256 inputs.
+cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, DeviceStatus *status, const TcOptions &opt,
+                         cudaStream_t s, int *launches)
+{
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const LargePlan plan = plan_large(A, sms);
+    const bool odd = tiles_of(A) % 2, off_cut = plan.off_slices > 1, tile_cut = plan.tile_slices > 1;
+    A.last_as_block = !tile_cut && last_tile_as_block(A, sms);
+    TcOptions add = opt;
+    add.add_after = fresh;
+    if (fresh && (off_cut || tile_cut)) {
+        e = launch_overlapping(zero_large_kernel, sms, 256, 0, *launches > 0, s, reinterpret_cast<int2 *>(A.acc), A.n,
+                               A.n_chan, plan.off_chans, int(tile_cut));
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    e = launch_xeng_pair(&A, 1, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+    if (e != cudaSuccess) return e;
+    ++*launches;
+    TcArray part[kTcMaxOffParts];
+    CUtensorMap maps[kTcMaxOffParts];
+    const int before = A.n_chan - plan.off_chans;
+    for (int cut = 0; cut <= int(off_cut); ++cut) {
+        const int count = cut ? plan.off_slices : 1;
+        if (cut) slices_of(A, before, plan.off_chans, count, part);
+        else part[0] = part_of(A, 0, before, 0, A.nt);
+        for (int k = 0; k < count; ++k) {
+            e = encode_map(part[k], &maps[k]);
+            if (e != cudaSuccess) return e;
+        }
+        e = launch_xeng_off(part, maps, count, fresh && !cut, zero_invalid, dev, status, cut ? add : opt, true, s);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    if (odd && !A.last_as_block) {
+        if (tile_cut) slices_of(A, 0, A.n_chan, plan.tile_slices, part);
+        else part[0] = A;
+        e = launch_xeng_tile(part, tile_cut ? plan.tile_slices : 1, fresh && !tile_cut, zero_invalid, dev, status,
+                             tile_cut ? add : opt, true, s);
+        *launches += e == cudaSuccess;
+    }
+    return e;
+}
+
 // The launches of the arrays of one mode, longest integrations first (a CTA's
 // last items are then its shortest).
 // The launches of one call write disjoint parts of the output and may overlap: each lets
@@ -186,12 +327,8 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     for (int x = 1; x < m; ++x)
         for (int y = x; y > 0 && sorted[y].nt > sorted[y - 1].nt; --y) std::swap(sorted[y], sorted[y - 1]);
     cudaError_t e = cudaSuccess;
-    if (count == 1 && m == 1) {
-        int sms = 0;
-        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        if (e != cudaSuccess) return e;
-        sorted[0].last_as_block = last_tile_as_block(sorted[0], sms);
-    }
+    if (count == 1 && m == 1 && sorted[0].n > 2 * kTile)
+        return launch_large(sorted[0], fresh, zero_invalid, dev, status, opt, s, launches);
     int n = 0;
     for (int k = 0; k < m; ++k)
         if (sorted[k].n > kTile) part[n++] = sorted[k];
@@ -212,7 +349,7 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     *launches += n > 0;
     n = 0;
     for (int k = 0; k < m; ++k)
-        if (tiles_of(sorted[k]) % 2 && !sorted[k].last_as_block) part[n++] = sorted[k];
+        if (tiles_of(sorted[k]) % 2) part[n++] = sorted[k];
     if (n) e = launch_blocks(false, part, n, count == 1 && part[0].n <= kTile, fresh, zero_invalid, dev, status, opt, s,
                              launches);
     return e;

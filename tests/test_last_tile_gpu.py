@@ -1,6 +1,7 @@
-"""The last of an odd number of tiles, alone or as a block with an empty second tile: channel
-counts on both sides of the rule that chooses, one input to a whole tile in it, stored, added
-and with the fused beam, bit-exact against the oracle."""
+"""Arrays of more than 256 inputs in one call.  The last of an odd number of tiles, alone or as
+a block with an empty second tile: channel counts on both sides of the rule that chooses, one
+input to a whole tile in it; long integrations whose last round of items goes in slices of
+samples.  Stored, added and with the fused beam, bit-exact against the oracle."""
 import numpy as np
 import pytest
 import torch
@@ -18,6 +19,20 @@ pytestmark = pytest.mark.gpu
                                    (257, 26, 70), (304, 51, 65), (384, 38, 64), (513, 11, 130), (640, 28, 63)])
 @pytest.mark.parametrize("zero_invalid", [False, True])
 def test_last_tile_exact(N, F, T, zero_invalid):
+    _check(N, F, T, zero_invalid)
+
+
+# few items of the tiles off the blocks left for the last round, with last tiles and without; last
+# tiles alone left for it; a last slice that ends within a stage; padded rows; two whole rounds
+@pytest.mark.parametrize("N,F,T,zero_invalid", [(512, 20, 5000, False), (400, 20, 4999, True), (512, 39, 4100, True),
+                                                (640, 13, 5057, False), (272, 38, 4300, True), (300, 37, 4097, False),
+                                                (257, 76, 6020, False), (768, 9, 4160, True), (1024, 5, 4200, False),
+                                                (520, 13, 4100, False)])
+def test_last_round_in_slices(N, F, T, zero_invalid):
+    _check(N, F, T, zero_invalid)
+
+
+def _check(N, F, T, zero_invalid):
     if not path_available("tc_fp8", N):
         pytest.skip("tc_fp8 unsupported")
     volt = np.random.default_rng(N + F + T).integers(0, 256, (T, F, N), dtype=np.uint8)
