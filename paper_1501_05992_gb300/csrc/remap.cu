@@ -34,8 +34,12 @@ constexpr int kRemapThreads = 256;
 constexpr int kRemapMaxDumps = 8;
 // Blocks of a launch, about: many, so that the last of them leave no gap (1600, 3200, 6400
 // and 12800 blocks: 166, 156, 150 and 148 us for the shape above), fewer where each of
-// them builds the table (512 inputs x 600 channels 198 us with 6400, 210 with 12800).
-constexpr int kRemapBlocks = 12800, kRemapTableBlocks = 6400;
+// them builds the table (512 inputs x 600 channels 198 us with 6400, 210 with 12800).  A thread
+// finds its station pair's elements once and loads four triples at a time, so no block has a
+// single group of one triple (256 inputs x 200, 300 and 400 channels 26.6 -> 20.5, 37.0 -> 29.1
+// and 47.2 -> 37.0 us, with two groups at least), nor of two unless blocks are few (256 x 600 / 2
+// 44.4 -> 39.2 us, but 128 x 600 / 2, 2700 blocks, 13.2 -> 14.3).
+constexpr int kRemapBlocks = 12800, kRemapTableBlocks = 6400, kRemapFewBlocks = 3200;
 
 struct RemapArgs {
     const int32_t *tri[kRemapMaxDumps];
@@ -146,7 +150,11 @@ cudaError_t launch_remap(const int32_t *const *tri, int n_dumps, int n, int n_ch
     const long long want = (Q + kRemapThreads - 1) / kRemapThreads;
     const int bx = int(want < 4096 ? want : 4096);
     const int groups = n_chan / f_avg;
-    const int rows = ((nat_of_pfb ? kRemapTableBlocks : kRemapBlocks) + bx - 1) / bx, by = groups < rows ? groups : rows;
+    int by = ((nat_of_pfb ? kRemapTableBlocks : kRemapBlocks) + bx - 1) / bx;
+    const int comb = n_dumps * f_avg;
+    const bool two = comb == 1 || (comb == 2 && (long long)groups * bx >= kRemapFewBlocks);
+    const int most = two ? (groups + 1) / 2 : groups;
+    if (by > most) by = most;
     const dim3 grid{unsigned(bx), unsigned(by)};
     if (nat_of_pfb)
         remap_kernel<true><<<grid, kRemapThreads, size_t(n) * sizeof(int), s>>>(args, n, n_chan, f_avg, nat_of_pfb, out);
