@@ -89,35 +89,20 @@ __device__ __forceinline__ uint32_t drop_invalid(uint32_t w)
     return w & ((t & (t >> 4) & 0x01010101u) * 0xFFu);
 }
 
-// Threads of a block and channels it takes, for kL lanes per row.  Small blocks leave
-// a shorter tail and need no more loads in flight than four per thread: 256 inputs x
-// 3072 channels x 500 samples 69.5 us with 256 threads and 128 channels, 66.3 with 128
-// and 64, 64.1 with 64 and 32 (59 us at the measured copy rate); rows of few lanes
-// gain nothing below 128 and 64.  Testing 16 samples at a time for invalid ones: 111
-// -> 92 us with one sample in eight invalid, 99 with smaller blocks and no such test.
-template <int kL>
-__host__ __device__ constexpr int beam_threads() { return kL >= 8 ? 64 : 128; }
-template <int kL>
-__host__ __device__ constexpr int beam_chans()
-{
-    const int groups = beam_threads<kL>() / kL, chans = kL >= 8 ? 32 : 64;
-    return groups > chans ? groups : chans;
-}
-
 // kL lanes per channel row (N a multiple of 16 kL; 16-byte aligned rows).  A
-// thread takes kU of its group's channels at a time, so that kU loads (per
-// chunk) are in flight before the first is used.
-template <bool kZeroInvalid, int kL>
-__global__ void __launch_bounds__(beam_threads<kL>())
+// block of kThreads takes kIter channels per group of lanes, a thread kU of them
+// at a time, so that kU loads (per chunk) are in flight before the first is used.
+// kEven: the blocks of a sample take `per` channels each instead of as many as they can.
+template <bool kZeroInvalid, int kL, int kThreads, int kIter, bool kEven>
+__global__ void __launch_bounds__(kThreads)
 beam_rows_kernel(const uint8_t *__restrict__ volt, int n, int n_chan, int n_avg, int n_out,
-                 int32_t *__restrict__ out)
+                 int32_t *__restrict__ out, int per)
 {
-    constexpr int kGroups = beam_threads<kL>() / kL, kChans = beam_chans<kL>();
-    constexpr int kIter = kChans / kGroups;
+    constexpr int kGroups = kThreads / kL, kChans = kGroups * kIter;
     constexpr int kU = kIter < 4 ? kIter : 4;
     const int sub = threadIdx.x % kL, group = threadIdx.x / kL;
     const int per_lane = n / (16 * kL);
-    const int f0 = blockIdx.x * kChans;
+    const int f0 = blockIdx.x * (kEven ? per : kChans), f1 = kEven ? min(n_chan, f0 + per) : n_chan;
     for (int k = blockIdx.y; k < n_out; k += gridDim.y) {
         // the trip counts are the same for every group, so whole warps shuffle
         for (int fb = group; fb < kChans; fb += kU * kGroups) {
@@ -128,9 +113,9 @@ beam_rows_kernel(const uint8_t *__restrict__ volt, int n, int n_chan, int n_avg,
                 const uint4 *row[kU];
 #pragma unroll
                 for (int u = 0; u < kU; ++u) {
-                    // a channel past the end reads channel 0's row and is not stored
+                    // a channel past the end reads another's row and is not stored
                     const int f = f0 + fb + u * kGroups;
-                    row[u] = reinterpret_cast<const uint4 *>(volt + ((size_t)t * n_chan + (f < n_chan ? f : 0)) * n) +
+                    row[u] = reinterpret_cast<const uint4 *>(volt + ((size_t)t * n_chan + (f < f1 ? f : kEven ? f0 : 0)) * n) +
                              sub;
                 }
                 int p[kU];
@@ -161,18 +146,58 @@ beam_rows_kernel(const uint8_t *__restrict__ volt, int n, int n_chan, int n_avg,
 #pragma unroll
                 for (int o = kL / 2; o >= 1; o /= 2) acc[u] += __shfl_xor_sync(0xFFFFFFFFu, acc[u], o);
                 const int f = f0 + fb + u * kGroups;
-                if (sub == 0 && f < n_chan) out[(size_t)k * n_chan + f] = acc[u];
+                if (sub == 0 && f < f1) out[(size_t)k * n_chan + f] = acc[u];
             }
         }
     }
 }
 
+template <bool kZeroInvalid, int kL, int kThreads, int kIter, bool kEven = false>
+void launch_blocks(const uint8_t *volt, int n, int n_chan, int n_avg, int n_out, int32_t *out, cudaStream_t s)
+{
+    // a few outputs per block: 1024 rows of blocks at most
+    const int blocks = div_up(n_chan, kThreads / kL * kIter), rows = n_out < 1024 ? n_out : 1024;
+    const dim3 grid{unsigned(blocks), unsigned(rows)};
+    beam_rows_kernel<kZeroInvalid, kL, kThreads, kIter, kEven>
+        <<<grid, kThreads, 0, s>>>(volt, n, n_chan, n_avg, n_out, out, div_up(n_chan, blocks));
+}
+
+// Threads of a block and channels it takes, for kL lanes per row.  Small blocks leave
+// a shorter tail and need no more loads in flight than four per thread: 256 inputs x
+// 3072 channels x 500 samples 69.5 us with 256 threads and 128 channels, 66.3 with 128
+// and 64, 64.1 with 64 and 32 (59 us at the measured copy rate).  Testing 16 samples at a
+// time for invalid ones: 111 -> 92 us with one sample in eight invalid, 99 with smaller
+// blocks and no such test.
+//  - 16 or 32 lanes: a thread's turns of four channels follow each other, so that few blocks
+//    are bound by latency.  One turn (8 channels of 32 lanes; 16 of 16 lanes up to six blocks
+//    of 32 per SM): 1024 inputs x 40 channels x 400 samples, ten added, 25.5 -> 9.1 us, 256 x 40 x
+//    400 / 10 11.1 -> 7.0; with more blocks 16 channels are slower (768 x 1500 x 300 / 10 60 us, 68).
+//  - 1 or 2 lanes: where a sample takes two blocks and the second is partly empty, the full
+//    ones land on every other SM; two of equal shares don't mind (1008 x 130 x 800 31.3 -> 19.3 us).
+//    Rows of up to 64 bytes by themselves are a load or two a thread and want bigger blocks
+//    (32 x 3072 x 800 23.4 -> 20.0 us).
 template <bool kZeroInvalid, int kL>
 void launch_rows(const uint8_t *volt, int n, int n_chan, int n_avg, int n_out, int32_t *out, cudaStream_t s)
 {
-    // a few outputs per block: 1024 rows of blocks at most
-    const dim3 grid(unsigned(div_up(n_chan, beam_chans<kL>())), unsigned(n_out < 1024 ? n_out : 1024));
-    beam_rows_kernel<kZeroInvalid, kL><<<grid, beam_threads<kL>(), 0, s>>>(volt, n, n_chan, n_avg, n_out, out);
+    constexpr long long kFewBlocks = 6 * 152;
+    if constexpr (kL <= 2) {
+        constexpr int kChans = 128 / kL;
+        if (n <= 64 && n_avg == 1)
+            launch_blocks<kZeroInvalid, kL, 256, 1>(volt, n, n_chan, n_avg, n_out, out, s);
+        else if (n_chan > kChans && n_chan < 2 * kChans)
+            launch_blocks<kZeroInvalid, kL, 128, 1, true>(volt, n, n_chan, n_avg, n_out, out, s);
+        else
+            launch_blocks<kZeroInvalid, kL, 128, 1>(volt, n, n_chan, n_avg, n_out, out, s);
+    } else if constexpr (kL == 4) {
+        launch_blocks<kZeroInvalid, kL, 128, 2>(volt, n, n_chan, n_avg, n_out, out, s);
+    } else if constexpr (kL == 16) {
+        if ((long long)div_up(n_chan, 32) * n_out <= kFewBlocks)
+            launch_blocks<kZeroInvalid, kL, 64, 4>(volt, n, n_chan, n_avg, n_out, out, s);
+        else
+            launch_blocks<kZeroInvalid, kL, 64, 8>(volt, n, n_chan, n_avg, n_out, out, s);
+    } else {
+        launch_blocks<kZeroInvalid, kL, 64, 4>(volt, n, n_chan, n_avg, n_out, out, s);
+    }
 }
 
 template <bool kZeroInvalid>
