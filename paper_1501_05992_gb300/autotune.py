@@ -4,11 +4,11 @@ For an array of N inputs x F channels x T samples per integration, every
 candidate (path, tile) the device supports is timed on a probe block of the
 same N and T (random bytes: the kernels' speed does not depend on the values)
 with a bounded number of channels, and the fastest is kept in a JSON cache
-keyed by device name and shape.  The candidates are the library's tile shapes
-(Section 3.4.2: the tile sets the arithmetic intensity): tcgen05 FP8, whose
-split into tiles is by shape (128 and 256 measure the same kernels); int8
-mma.sync on 64 x 64; and the dp4a CUDA-core kernel on 64 x 64 or
-32 x 32 tiles.
+keyed by device name, shape, library version and candidates.  The candidates
+are the library's tile shapes (Section 3.4.2: the tile sets the arithmetic
+intensity): tcgen05 FP8, whose split into tiles is by shape; int8 mma.sync on
+64 x 64; and the CUDA-core path by shape (tile 0: up to 64 inputs the kernel
+of 4 x 4 tiles, else 64 x 64) or with 64 x 64 or 32 x 32 tiles of dp4a.
 """
 from __future__ import annotations
 
@@ -20,12 +20,15 @@ import torch
 
 from . import corr
 
-CANDIDATES = [("tc_fp8", 256), ("tc_fp8", 128), ("mma_i8", 0), ("cudacore", 64), ("cudacore", 32)]
+CANDIDATES = [("tc_fp8", 0), ("mma_i8", 0), ("cudacore", 0), ("cudacore", 64), ("cudacore", 32)]
 _lock = threading.Lock()
 
 
-def _key(device: torch.device, n_inputs: int, n_chan: int, n_time: int) -> str:
-    return f"{torch.cuda.get_device_name(device)}|{n_inputs}x{n_chan}x{n_time}"
+def _key(device: torch.device, n_inputs: int, n_chan: int, n_time: int, candidates=CANDIDATES) -> str:
+    # what a result was chosen from belongs to it: with other kernels or candidates it is no answer
+    forms = ",".join(f"{path}/{tile}" for path, tile in candidates)
+    return (f"{torch.cuda.get_device_name(device)}|{n_inputs}x{n_chan}x{n_time}"
+            f"|v{corr.load().corr_version()}|{forms}")
 
 
 def _load(path: str | None) -> dict:
@@ -53,7 +56,7 @@ def tune(n_inputs: int, n_chan: int, n_time: int, cache_path: str | None = None,
     """Fastest (path, tile) for the shape: {"path", "tile", "ms": {...}}."""
     dev = torch.device("cuda", torch.cuda.current_device() if device is None else
                        (device if isinstance(device, int) else device.index or 0))
-    key = _key(dev, n_inputs, n_chan, n_time)
+    key = _key(dev, n_inputs, n_chan, n_time, candidates)
     with _lock:
         cache = _load(cache_path)
         if key in cache:
