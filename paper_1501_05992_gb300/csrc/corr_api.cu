@@ -89,11 +89,11 @@ struct WsLayout {
 };
 
 // Row stride of the tensor-core path's padded copy, and the samples one copy
-// holds (0 when the rows need no padding).
+// holds (0 when the rows need no padding, or the kernel reads them as they are).
 int tc_ld(int n) { return int(round_up(size_t(n), 16)); }
 int tc_pad_samples(int n, int n_chan, int t_max)
 {
-    if (n % 16 == 0) return 0;
+    if (n % 16 == 0 || tc_any_rows(n)) return 0;
     const size_t row = size_t(tc_ld(n)) * size_t(n_chan);
     size_t t = kTcPadCap / row / 64 * 64;
     if (t < 64) t = 64;
@@ -207,10 +207,9 @@ int accumulate_to(corr_ctx *c, const uint8_t *volt, int nt, int32_t *target, boo
     cudaError_t e = cudaSuccess;
     const size_t row = size_t(c->f) * size_t(c->n);
     if (path == CORR_PATH_TC_FP8) {
-        // rows of n % 16 != 0 inputs go through a padded copy, chunk by chunk, except
-        // where the kernel reads them as they are
+        // rows that need it go through a padded copy, chunk by chunk
         if (c->n % 16 == 0 && (reinterpret_cast<uintptr_t>(volt) & 15) != 0) return CORR_E_ARG;
-        const int pad_t = tc_any_rows(c->n) ? 0 : tc_pad_samples(c->n, c->f, c->t_max);
+        const int pad_t = tc_pad_samples(c->n, c->f, c->t_max);
         const int step = pad_t ? (pad_t < kTcMaxSamples ? pad_t : kTcMaxSamples) : kTcMaxSamples;
         for (int t0 = 0; t0 < nt; t0 += step) {
             const int ntc = nt - t0 < step ? nt - t0 : step;
