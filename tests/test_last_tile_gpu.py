@@ -48,3 +48,28 @@ def _check(N, F, T, zero_invalid):
     assert np.array_equal(tri.cpu().numpy(), oracle.to_int32(vis))
     assert np.array_equal(acc.cpu().numpy(), oracle.to_int32(2 * vis))
     assert np.array_equal(beam.cpu().numpy(), oracle.beam(volt, 1, zero_invalid))
+
+
+def test_slices_under_capture():
+    """The launches of a call in slices, which overlap and wait for the zeroing, replayed from a
+    graph on new samples and twice in a row."""
+    N, F, T = 640, 13, 4200
+    if not path_available("tc_fp8", N):
+        pytest.skip("tc_fp8 unsupported")
+    b = corr.Batch([dict(n_inputs=N, n_chan=F, n_time_per_int=T, path="tc_fp8")])
+    rng = np.random.default_rng(5)
+    volt = rng.integers(0, 256, (T, F, N), dtype=np.uint8)
+    d = torch.from_numpy(volt).cuda()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    graph, outs = b.capture([d], stream=stream)
+    for _ in range(2):
+        d.copy_(torch.from_numpy(volt))
+        torch.cuda.synchronize()
+        graph.launch(stream)
+        graph.launch(stream)
+        stream.synchronize()
+        assert np.array_equal(outs[0].cpu().numpy(), oracle.to_int32(oracle.xmac(volt)))
+        volt = rng.integers(0, 256, (T, F, N), dtype=np.uint8)
+    b.sync(stream)
+    graph.close()
