@@ -307,14 +307,15 @@ def load_peaks():
                 "sm_max_mhz": 2070.0}, "fallback"
 
 
-def measured_traffic(kernel_src: str, profile_md: str, workload: str):
+def measured_traffic(sources: list[str], profile_md: str, workload: str):
     """DRAM bytes per integration from the committed ncu summary, but only while the
-    kernel source still matches the one the counters were taken from."""
+    sources (the kernel's and the one that splits a call into its launches) still match
+    those that the counters were taken from."""
     import hashlib
     import re
     try:
         text = open(profile_md).read()
-        sha = hashlib.sha256(open(kernel_src, "rb").read()).hexdigest()[:16]
+        sha = hashlib.sha256(b"".join(open(s, "rb").read() for s in sources)).hexdigest()[:16]
     except OSError:
         return None
     m = re.search(r"sha256 prefix `([0-9a-f]{16})`", text)
@@ -551,7 +552,7 @@ def measure_beam_fused(n, f, t, volt, stream_, dev):
 
 def measure_uneven_batch(stream_, dev, peaks, sm_count):
     """The uneven batch (three arrays of 128, 256 and 1024 inputs) correlated
-    in one persistent launch, each array's path chosen by the autotuner:
+    in one call, each array's path chosen by the autotuner:
     whole-batch and per-array throughput, and whole triangles of two channels
     of every array against the oracle (the 1024-input array at its full
     10000 samples)."""
@@ -830,7 +831,8 @@ def run_ours(args, world, rank, local):
     avg_ms = xe_ms / max(1, xe_timed)
     main_path = paths[max(range(len(arrays)), key=lambda a: arrays[a][0] ** 2 * arrays[a][1] * arrays[a][2])]
     roof = roofline_for(main_path, ops_per_launch, avg_ms, peaks, src, sm_count, measured_probes(dev))
-    traffic = (measured_traffic(os.path.join(ROOT, "paper_1501_05992_gb300", "csrc", "xeng_diag.cuh"),
+    csrc = os.path.join(ROOT, "paper_1501_05992_gb300", "csrc")
+    traffic = (measured_traffic([os.path.join(csrc, f) for f in ("xeng_diag.cuh", "xeng_tc.cu")],
                                 os.path.join(ROOT, "profiles", "xeng_pair_full_band_traffic.md"),
                                 args.workload) if main_path == "tc_fp8" else None)
     roof["traffic"] = traffic * n_int / max(1, xe_per_step) if traffic else None    # per launch

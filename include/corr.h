@@ -114,7 +114,7 @@ int corr_set_path(corr_ctx *ctx, int path);
 /* Tile shape (Section 3.4.2, Eq. 4: the tile sets the arithmetic intensity).
  * CUDA-core path: 32 or 64 inputs per side, or 0 to choose by shape: a kernel
  * of 4 x 4 tiles without operand staging up to 64 inputs and 65535 channels,
- * else 64.  128 and 256 are accepted for the tcgen05 path, which chooses its
+ * else 64 (32 for up to 32 inputs).  128 and 256 are accepted for the tcgen05 path, which chooses its
  * work items itself (256-input blocks on the diagonal, the tiles off them, a
  * last tile alone); no value changes it.  Any other value: CORR_E_ARG.  Only
  * between integrations (CORR_E_STATE). */

@@ -951,10 +951,10 @@ corr_ctx *corr_batch_array(corr_batch *b, int a)
 namespace {
 
 // Correlate every array of a batch that has data: tensor-core arrays in persistent
-// launches of groups of up to CORR_BATCH_TC_GROUP arrays, per kTcMaxSamples samples, the others on their own kernels.  With `into` null
-// the samples are added to the arrays' running integrations; otherwise each
-// array's whole integration is written to into[a] (its accumulators are left
-// alone).
+// launches of groups of up to CORR_BATCH_TC_GROUP arrays, per kTcMaxSamples
+// samples, the others on their own kernels.  With `into` null the samples are
+// added to the arrays' running integrations; otherwise each array's whole
+// integration is written to into[a] (its accumulators are left alone).
 int batch_correlate(corr_batch *b, const uint8_t *const *d_volt, const int *n_time, int32_t *const *into,
                     cudaStream_t s)
 {

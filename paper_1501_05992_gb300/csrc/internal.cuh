@@ -67,8 +67,8 @@ cudaError_t launch_unpack_kmajor(const uint8_t *volt, int n_chan, int n, int f0,
                                  int8_t *out, int8_t *out_tw, cudaStream_t s);
 
 // Copy `rows` rows of n bytes (stride n in src) to a stride of ld >= n bytes
-// in dst (the tensor-core path's 16-byte row alignment); bytes between rows
-// are left as they are.
+// in dst (the tensor-core path's 16-byte row alignment).  Bytes between rows
+// become zero, i.e. samples 0 + 0i: the kernels read the last piece of a row whole.
 cudaError_t launch_pad_rows(const uint8_t *src, long long rows, int n, int ld, uint8_t *dst, cudaStream_t s);
 
 // CUDA-core X-engine over a staged channel chunk; adds (or, if `fresh`,

@@ -20,8 +20,10 @@
 // The tensor-core path reads the packed bytes themselves.  Beyond 256 inputs they come
 // through TMA, which needs rows (the n inputs of one channel and sample) that start on
 // 16-byte boundaries.  For other input counts the rows are first copied to a stride
-// of round_up(n, 16) bytes (the bytes between rows are never read: the
-// tensor map's extent is n and TMA fills columns past it with zeros).
+// of round_up(n, 16) bytes.  The bytes between rows must be zero: the tensor map's
+// extent is n, so that TMA fills the columns past it with zeros by itself, but the
+// blocks on the diagonal are read as whole 16-byte pieces, and the fused beam adds
+// up the power of every byte of a piece.
 #include "decode.cuh"
 #include "internal.cuh"
 

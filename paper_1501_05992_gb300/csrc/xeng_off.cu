@@ -3,17 +3,23 @@
 //
 // One work item is (channel, tile I of 128 inputs, block J of 256 inputs left of
 // I's own block): two 128 x 128 tiles of the triangle.  CTA r of the pair takes
-// tile r of J as its 128 accumulator rows, and both take I as the columns in the
-// [Re | Im] form of xeng_tc.cu: with u = v + 8 (E4M3 bit pattern u, value u * 2^-9),
+// tile r of J as its 128 accumulator rows, and both take I as the columns in [Re | Im]
+// form: 128 columns of real parts, then 128 of imaginary ones.  The operands are the
+// nibbles' codes u = v + 8 (0..15; the E4M3 bit pattern u has the value u * 2^-9),
 //
 //   D += R_J . [R_I | -M_I],   D += M_J . [M_I | R_I]
+//
+// so that the accumulator times 2^18 is an integer below 2^24 and exact.  It differs
+// from the product of the samples by terms in each input's sums of codes alone: with
+// E = sum(ur + um) and D = sum(um - ur) over the T samples (those past the end have
+// code 8), Re V_ij = P_re - 8 E_i - 8 E_j + 128 T and Im V_ij = -P_im - 8 D_i + 8 D_j.
 //
 // where the two halves of the 256 columns are the two CTAs' shares of the MMA's B
 // operand: CTA 0 converts I into (R, M), CTA 1 into (-M, R), each J tile into
 // (R, M).  A pair of SMs so reads 8 KB of operands per M=256 N=256 K=32 MMA and SM
 // where one SM alone (M=128) reads 12 KB, and converts each I tile into two planes
-// instead of three.  The offsets are corrected in the epilogue from per-input sums
-// (as in xeng_tc.cu), which every CTA has for both of its tiles.
+// instead of three.  The converters add the codes up on their way, so that every CTA has
+// the sums of both of its tiles, and the epilogue takes the terms off.
 //
 // Roles per CTA: warps 0-7 epilogue (two per quarter of the accumulator's lanes),
 // warps 8-23 converters (two teams of eight that take alternate 64-sample stages;

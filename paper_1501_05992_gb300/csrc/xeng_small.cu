@@ -1,4 +1,4 @@
-// X-engine for small arrays (n < 64 inputs) on the CUDA cores, straight from the
+// X-engine for small arrays (up to 64 inputs) on the CUDA cores, straight from the
 // packed voltages.
 //
 // The same dp4a form as xeng_dp4a.cu (two samples of a complex product per

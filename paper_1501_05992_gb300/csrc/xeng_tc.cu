@@ -8,7 +8,8 @@
 //     inputs is nothing else): single CTAs, xeng_tile.cu, or a block whose second tile is
 //     empty (last_tile_as_block);
 //   - the tiles off those blocks, from 257 inputs on: CTA pairs, xeng_off.cu.
-// Each is one persistent launch over every channel of up to kTcMaxArrays arrays.
+// Each is one persistent launch over every channel of up to kTcMaxArrays arrays; a call of
+// one array may cut its last round into slices of samples, which take launches of their own.
 // Whether invalid samples are zeroed (CORR_ZERO_INVALID) and whether the launch stores
 // or adds are properties of the kernel, so arrays that differ in them go to different
 // launches.
@@ -70,7 +71,7 @@ cudaError_t encode_map(const TcArray &A, CUtensorMap *map)
 // per channel, 0.42 us: a slice has 16 at least (about what its stores take), and splitting
 // costs the zeroing, the adds and a launch, more where it is a second launch (about 14 and
 // 26).  256 inputs x 5000 samples: 4 channels 39.7 -> 21.3 us, 80 channels 72 -> 60 us,
-// 768 channels 359 -> 345 us (with the beam 393 -> 375); 40 channels x 20000 samples 125 ->
+// 768 channels 359 -> 345 us (with the beam 401 -> 390); 40 channels x 20000 samples 125 ->
 // 94 us; 16 x 2200 24.9 -> 20.9 us.  128 inputs x 5000 samples: 40 channels 37.5 -> 20.9 us,
 // 160 channels 68 -> 52 us, 768 channels 188 -> 171 us.
 constexpr int kSplitCost = 26, kSplitCostAlone = 14;
@@ -315,7 +316,7 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
 // The launches of one call write disjoint parts of the output and may overlap: each lets
 // the next one's CTAs take the SMs as its own leave them (in place of an empty last round
 // per launch: 384 inputs x 384 channels x 5000 samples 0.51 -> 0.45 ms, 1024 x 128 x 10000
-// 1.81 -> 1.74 ms), and ends only when the one before has.
+// 1.81 -> 1.73 ms), and ends only when the one before has.
 cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero_invalid, int dev,
                          DeviceStatus *status, const TcOptions &opt, cudaStream_t s, int *launches)
 {
