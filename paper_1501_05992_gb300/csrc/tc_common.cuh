@@ -1,4 +1,4 @@
-// Device helpers shared by the tensor-core X-engines (xeng_diag.cuh, xeng_off.cu):
+// Device helpers shared by the tensor-core X-engines (xeng_diag.cuh, xeng_off.cuh):
 // mbarriers with bounded waits, TMA, tcgen05 and the decoding of packed samples.
 #pragma once
 
@@ -381,9 +381,13 @@ cudaError_t launch_xeng_pair(const TcArray *arrays, int count, bool fresh, bool 
                              DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
 cudaError_t launch_xeng_tile(const TcArray *arrays, int count, bool fresh, bool zero_invalid, int dev,
                              DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
-// The rest of their triangles (xeng_off.cu), for arrays of 257 or more inputs;
+// The rest of their triangles (xeng_off.cuh), for arrays of 257 or more inputs;
 // maps[k] is array k's tensor map (boxes of 128 inputs x 1 channel x 64 samples).
 cudaError_t launch_xeng_off(const TcArray *arrays, const CUtensorMap *maps, int count, bool fresh, bool zero_invalid,
                             int dev, DeviceStatus *status, const TcOptions &opt, bool overlap, cudaStream_t s);
+// Both for one array, on pairs of CTAs of their own each.
+cudaError_t launch_xeng_both(const TcArray &A, const CUtensorMap &map, int block_pairs, int off_pairs, bool fresh,
+                             bool zero_invalid, int dev, DeviceStatus *status, const TcOptions &opt, bool overlap,
+                             cudaStream_t s);
 
 }  // namespace corr

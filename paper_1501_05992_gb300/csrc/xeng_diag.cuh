@@ -20,7 +20,7 @@
 // and V is Hermitian, so W[b][a] = Re V_ab + Im V_ab: W holds every product of
 // the block once, Re V_ij = (W[j][i] + W[i][j]) / 2 and Im V_ij = (W[j][i] -
 // W[i][j]) / 2.  That is two real products per pair of 128-input tiles and
-// none wasted, where a diagonal tile in [Re | Im] form (xeng_off.cu) computes
+// none wasted, where a diagonal tile in [Re | Im] form (xeng_off.cuh) computes
 // four and throws half of them away: 8 tile products per 256 inputs against 12.
 //
 // Encoding (exact): the three planes q in [-15, 15], r in [-8, 7] and 2 m in
@@ -217,8 +217,10 @@ __device__ __forceinline__ uint4 load16(const uint8_t *a)
     return v;
 }
 
-template <bool kPair, bool kAligned, bool kFresh, bool kZeroInvalid, bool kBeam>
-__device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
+// The items first_item, first_item + item_step, ... of a launch, by this CTA or pair of CTAs.
+// kSpareWarps: the block has more warps than the roles take.
+template <bool kPair, bool kAligned, bool kFresh, bool kZeroInvalid, bool kBeam, bool kSpareWarps = false>
+__device__ __forceinline__ void block_body(const Params &p, uint8_t *smem, int first_item, int item_step)
 {
     const uint32_t sbase = smem_u32(smem);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -265,7 +267,6 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
     fence_after();
     const uint32_t tmem = *tmem_slot;
     let_next_launch_start();
-    const int first_item = blockIdx.x >> (kPair ? 1 : 0), item_step = gridDim.x >> (kPair ? 1 : 0);
 
     if (warp == kMmaWarp) {
         // ------------------------------------- MMA issuer (leader CTA) --
@@ -333,6 +334,8 @@ __device__ __forceinline__ void block_body(const Params &p, uint8_t *smem)
             while (!mbar_try(bar_drain, 0) && clock64() - t0 < p.drain_limit) {
             }
         }
+    } else if (kSpareWarps && warp > kMmaWarp) {
+        // nothing to do
     } else if (warp >= kFirstConvWarp) {
         // ----------------------------------------------------- converters --
         // Team t converts the stages g (counted over all items of this CTA) with

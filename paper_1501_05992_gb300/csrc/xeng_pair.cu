@@ -9,7 +9,7 @@ template <bool kAligned, bool kFresh, bool kZeroInvalid, bool kBeam>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1) xeng_pair_kernel(const __grid_constant__ Params p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    block_body<true, kAligned, kFresh, kZeroInvalid, kBeam>(p, smem);
+    block_body<true, kAligned, kFresh, kZeroInvalid, kBeam>(p, smem, blockIdx.x >> 1, gridDim.x >> 1);
 }
 
 // [aligned][fresh][zero_invalid][beam]

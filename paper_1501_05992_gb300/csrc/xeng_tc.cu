@@ -7,7 +7,8 @@
 //   - the last tile alone, where the number of tiles is odd (an array of up to 128
 //     inputs is nothing else): single CTAs, xeng_tile.cu, or a block whose second tile is
 //     empty (last_tile_as_block);
-//   - the tiles off those blocks, from 257 inputs on: CTA pairs, xeng_off.cu.
+//   - the tiles off those blocks, from 257 inputs on: CTA pairs, xeng_off.cu; in few
+//     rounds both kinds go in one launch, xeng_both.cu.
 // Each is one persistent launch over every channel of up to kTcMaxArrays arrays; a call of
 // one array may cut its last round into slices of samples, which take launches of their own.
 // Whether invalid samples are zeroed (CORR_ZERO_INVALID) and whether the launch stores
@@ -246,6 +247,41 @@ LargePlan plan_large(const TcArray &A, int sms)
     return plan;
 }
 
+// Whether the blocks and the tiles off them go in one launch, with the pairs of CTAs divided
+// between the two kinds of items, and how: up to four rounds, where it takes no round more
+// than all items together.  A CTA then has its next item's samples and MMAs behind the stores
+// of the one before, where a second launch's CTA starts from nothing: 512 inputs x 38 channels
+// x 100, 300 and 1000 samples 20.8 -> 18.5, 24.6 -> 19.7 and 32.8 -> 25.5 us, 1024 x 8 x 1000
+// 32.7 -> 24.8, 640 x 32 x 300 30.8 -> 24.3, 512 x 60 x 1000 (four rounds) 47.3 -> 41.0.  With
+// more rounds long integrations lose (512 x 152 x 6000, eight rounds, 333 -> 346 us): power
+// bounds them, and one kind's pairs end before the other's.  The last of an odd number of
+// tiles goes with the blocks where that takes no round more (A.last_as_block); where it does,
+// only calls of one round go in one launch, since its own launch then fills the pairs that a
+// second round leaves idle (384 x 52 x 5000 81 us, 99 with both kinds in one launch).
+constexpr int kBothRounds = 4;
+
+bool one_launch(TcArray &A, int sms, int *block_pairs, int *off_pairs)
+{
+    const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2;
+    if (pairs < 2) return false;
+    const long long blocks = (long long)A.n_chan * half,
+                    offs = (long long)A.n_chan * (tiles % 2 ? half * half : half * (half - 1));
+    const int rounds = rounds_of(blocks + offs, pairs);
+    auto divide = [&](long long with_blocks) {
+        *block_pairs = rounds_of(with_blocks, rounds);
+        *off_pairs = rounds_of(offs, rounds);
+        return *block_pairs + *off_pairs <= pairs;
+    };
+    if (rounds > kBothRounds) return false;
+    if (tiles % 2 && divide(blocks + A.n_chan)) {
+        A.last_as_block = true;
+        return true;
+    }
+    if (!divide(blocks) || (tiles % 2 && rounds > 1)) return false;
+    A.last_as_block = false;
+    return true;
+}
+
 // Zeroes what the slices of a plan add to: for the last `chans` channels the elements left of
 // each row's own 256-input block, and (tiles) every channel's last tile.  A warp per row.
 __global__ void __launch_bounds__(256) zero_large_kernel(int2 *__restrict__ out, int n, int n_chan, int chans, int tiles)
@@ -275,6 +311,19 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
     const LargePlan plan = plan_large(A, sms);
     const bool odd = tiles_of(A) % 2, off_cut = plan.off_slices > 1, tile_cut = plan.tile_slices > 1;
     A.last_as_block = !tile_cut && last_tile_as_block(A, sms);
+    // few rounds of whole items: one launch
+    int block_pairs = 0, off_pairs = 0;
+    if (!off_cut && !tile_cut && one_launch(A, sms, &block_pairs, &off_pairs)) {
+        CUtensorMap map;
+        e = encode_map(A, &map);
+        if (e == cudaSuccess)
+            e = launch_xeng_both(A, map, block_pairs, off_pairs, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+        *launches += e == cudaSuccess;
+        if (e != cudaSuccess || !odd || A.last_as_block) return e;
+        e = launch_xeng_tile(&A, 1, fresh, zero_invalid, dev, status, opt, true, s);
+        *launches += e == cudaSuccess;
+        return e;
+    }
     TcOptions add = opt;
     add.add_after = fresh;
     if (fresh && (off_cut || tile_cut)) {

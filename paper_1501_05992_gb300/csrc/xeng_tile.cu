@@ -9,7 +9,7 @@ template <bool kAligned, bool kFresh, bool kZeroInvalid, bool kBeam>
 __global__ void __launch_bounds__(kThreads, 1) xeng_tile_kernel(const __grid_constant__ Params p)
 {
     extern __shared__ __align__(1024) uint8_t smem[];
-    block_body<false, kAligned, kFresh, kZeroInvalid, kBeam>(p, smem);
+    block_body<false, kAligned, kFresh, kZeroInvalid, kBeam>(p, smem, blockIdx.x, gridDim.x);
 }
 
 // [aligned][fresh][zero_invalid][beam]

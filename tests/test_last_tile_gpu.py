@@ -22,6 +22,15 @@ def test_last_tile_exact(N, F, T, zero_invalid):
     _check(N, F, T, zero_invalid)
 
 
+# one to four rounds of both kinds of items in one launch, one round with the last tiles apart, and
+# five rounds in launches of their own
+@pytest.mark.parametrize("N,F,T", [(512, 38, 70), (768, 20, 65), (1024, 14, 64), (400, 60, 63), (1024, 1, 200),
+                                   (640, 32, 130), (640, 12, 65), (500, 45, 64), (512, 95, 65)])
+@pytest.mark.parametrize("zero_invalid", [False, True])
+def test_both_kinds_of_items_in_one_launch(N, F, T, zero_invalid):
+    _check(N, F, T, zero_invalid)
+
+
 # few items of the tiles off the blocks left for the last round, with last tiles and without; last
 # tiles alone left for it; a last slice that ends within a stage; padded rows; two whole rounds
 @pytest.mark.parametrize("N,F,T,zero_invalid", [(512, 20, 5000, False), (400, 20, 4999, True), (512, 39, 4100, True),
