@@ -6,7 +6,7 @@
 //     xeng_pair.cu;
 //   - the last tile alone, where the number of tiles is odd (an array of up to 128
 //     inputs is nothing else): single CTAs, xeng_tile.cu, or a block whose second tile is
-//     empty (last_tile_as_block);
+//     empty (one_launch);
 //   - the tiles off those blocks, from 257 inputs on: CTA pairs, xeng_off.cu; in few
 //     rounds both kinds go in one launch, xeng_both.cu.
 // Each is one persistent launch over every channel of up to kTcMaxArrays arrays; a call of
@@ -166,20 +166,44 @@ cudaError_t launch_blocks(bool pair, const TcArray *arrays, int count, bool alon
 
 int tiles_of(const TcArray &A) { return (A.n + kTile - 1) / kTile; }
 
-// Whether the last tile of an array with an odd number of tiles, more than two, goes to the
-// pair kernel as a block whose second tile is empty: where the pairs of CTAs that its items
-// take are idle in the last round of the others, of two at most.  It saves the third launch
-// of a call (2 us of the host's time, and its start) and costs nothing then: 384 inputs x 20
-// channels x 100 samples 14.2 -> 12.4 us, 384 x 40 x 1000 32.8 -> 30.8, 640 x 20 x 100 22.6 ->
-// 20.6, 896 x 9 x 200 24.5 -> 22.6.  With a round more it is slower (384 x 26 x 1000 18.8 ->
-// 28.9 us), and with three rounds on short integrations (640 x 28 x 100 24.7 -> 26.7).
-bool last_tile_as_block(const TcArray &A, int sms)
+int rounds_of(long long items, int workers) { return int((items + workers - 1) / workers); }
+
+// Whether the blocks and the tiles off them go in one launch, with the pairs of CTAs divided
+// between the two kinds of items, and how: up to four rounds, where it takes no round more
+// than all items together.  A CTA then has its next item's samples and MMAs behind the stores
+// of the one before, where a second launch's CTA starts from nothing: 512 inputs x 38 channels
+// x 100, 300 and 1000 samples 20.8 -> 18.5, 24.6 -> 19.7 and 32.8 -> 25.5 us, 1024 x 8 x 1000
+// 32.7 -> 24.8, 640 x 32 x 300 30.8 -> 24.3, 512 x 60 x 1000 (four rounds) 47.3 -> 41.0.  With
+// more rounds long integrations lose (512 x 152 x 6000, eight rounds, 333 -> 346 us): power
+// bounds them, and one kind's pairs end before the other's.  The last of an odd number of
+// tiles goes with the blocks, as one whose second tile is empty, where that takes no round
+// more (384 x 20 x 100, a launch less, 14.2 -> 12.4 us); where it does, only calls of one round
+// go in one launch, since its own launch then fills the pairs that a second round leaves idle
+// (384 x 52 x 5000 81 us, 99 with both kinds in one launch).
+constexpr int kBothRounds = 4;
+
+struct OneLaunch {
+    bool fits = false, last_as_block = false;
+    int block_pairs = 0, off_pairs = 0;
+};
+
+OneLaunch one_launch(const TcArray &A, int sms)
 {
+    OneLaunch l;
     const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2;
-    if (tiles % 2 == 0 || tiles == 1 || pairs < 1) return false;
-    const long long others = (long long)A.n_chan * (half + half * half);     // blocks, and the tiles off them
-    const long long rounds = (others + pairs - 1) / pairs;
-    return rounds <= 2 && others + A.n_chan <= rounds * pairs;
+    if (pairs < 2) return l;
+    const long long blocks = (long long)A.n_chan * half,
+                    offs = (long long)A.n_chan * (tiles % 2 ? half * half : half * (half - 1));
+    const int rounds = rounds_of(blocks + offs, pairs);
+    auto divide = [&](long long with_blocks) {
+        l.block_pairs = rounds_of(with_blocks, rounds);
+        l.off_pairs = rounds_of(offs, rounds);
+        return l.block_pairs + l.off_pairs <= pairs;
+    };
+    if (rounds > kBothRounds) return l;
+    l.last_as_block = tiles % 2 && divide(blocks + A.n_chan);
+    l.fits = l.last_as_block || (divide(blocks) && (tiles % 2 == 0 || rounds == 1));
+    return l;
 }
 
 // The last round of a call of one array of more than 256 inputs.  Its items, the blocks and the
@@ -199,8 +223,6 @@ struct LargePlan {
 };
 constexpr int kLargeSplitCost = 20;
 
-int rounds_of(long long items, int workers) { return int((items + workers - 1) / workers); }
-
 LargePlan plan_large(const TcArray &A, int sms)
 {
     LargePlan plan;
@@ -208,7 +230,7 @@ LargePlan plan_large(const TcArray &A, int sms)
     if (pairs < 1) return plan;
     const int per_off = tiles % 2 ? half * half : half * (half - 1);
     const long long items = (long long)A.n_chan * (half + per_off);
-    const int lone = tiles % 2 && !last_tile_as_block(A, sms) ? A.n_chan : 0;       // last tiles alone
+    const int lone = tiles % 2 && !one_launch(A, sms).last_as_block ? A.n_chan : 0;       // last tiles alone
     const int full = int(items / pairs), left = int(items % pairs);
     const int whole = rounds_of(items, pairs), idle = left ? sms - 2 * left : 0;
     // whole items; the last tiles take the SMs that the last round leaves idle first
@@ -247,41 +269,6 @@ LargePlan plan_large(const TcArray &A, int sms)
     return plan;
 }
 
-// Whether the blocks and the tiles off them go in one launch, with the pairs of CTAs divided
-// between the two kinds of items, and how: up to four rounds, where it takes no round more
-// than all items together.  A CTA then has its next item's samples and MMAs behind the stores
-// of the one before, where a second launch's CTA starts from nothing: 512 inputs x 38 channels
-// x 100, 300 and 1000 samples 20.8 -> 18.5, 24.6 -> 19.7 and 32.8 -> 25.5 us, 1024 x 8 x 1000
-// 32.7 -> 24.8, 640 x 32 x 300 30.8 -> 24.3, 512 x 60 x 1000 (four rounds) 47.3 -> 41.0.  With
-// more rounds long integrations lose (512 x 152 x 6000, eight rounds, 333 -> 346 us): power
-// bounds them, and one kind's pairs end before the other's.  The last of an odd number of
-// tiles goes with the blocks where that takes no round more (A.last_as_block); where it does,
-// only calls of one round go in one launch, since its own launch then fills the pairs that a
-// second round leaves idle (384 x 52 x 5000 81 us, 99 with both kinds in one launch).
-constexpr int kBothRounds = 4;
-
-bool one_launch(TcArray &A, int sms, int *block_pairs, int *off_pairs)
-{
-    const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2;
-    if (pairs < 2) return false;
-    const long long blocks = (long long)A.n_chan * half,
-                    offs = (long long)A.n_chan * (tiles % 2 ? half * half : half * (half - 1));
-    const int rounds = rounds_of(blocks + offs, pairs);
-    auto divide = [&](long long with_blocks) {
-        *block_pairs = rounds_of(with_blocks, rounds);
-        *off_pairs = rounds_of(offs, rounds);
-        return *block_pairs + *off_pairs <= pairs;
-    };
-    if (rounds > kBothRounds) return false;
-    if (tiles % 2 && divide(blocks + A.n_chan)) {
-        A.last_as_block = true;
-        return true;
-    }
-    if (!divide(blocks) || (tiles % 2 && rounds > 1)) return false;
-    A.last_as_block = false;
-    return true;
-}
-
 // Zeroes what the slices of a plan add to: for the last `chans` channels the elements left of
 // each row's own 256-input block, and (tiles) every channel's last tile.  A warp per row.
 __global__ void __launch_bounds__(256) zero_large_kernel(int2 *__restrict__ out, int n, int n_chan, int chans, int tiles)
@@ -310,16 +297,16 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
     if (e != cudaSuccess) return e;
     const LargePlan plan = plan_large(A, sms);
     const bool odd = tiles_of(A) % 2, off_cut = plan.off_slices > 1, tile_cut = plan.tile_slices > 1;
-    A.last_as_block = !tile_cut && last_tile_as_block(A, sms);
-    // few rounds of whole items: one launch
-    int block_pairs = 0, off_pairs = 0;
-    if (!off_cut && !tile_cut && one_launch(A, sms, &block_pairs, &off_pairs)) {
+    const OneLaunch one = one_launch(A, sms);
+    if (one.fits && !off_cut && !tile_cut) {
+        A.last_as_block = one.last_as_block;
         CUtensorMap map;
         e = encode_map(A, &map);
         if (e == cudaSuccess)
-            e = launch_xeng_both(A, map, block_pairs, off_pairs, fresh, zero_invalid, dev, status, opt, *launches > 0, s);
+            e = launch_xeng_both(A, map, one.block_pairs, one.off_pairs, fresh, zero_invalid, dev, status, opt,
+                                 *launches > 0, s);
         *launches += e == cudaSuccess;
-        if (e != cudaSuccess || !odd || A.last_as_block) return e;
+        if (e != cudaSuccess || !odd || one.last_as_block) return e;
         e = launch_xeng_tile(&A, 1, fresh, zero_invalid, dev, status, opt, true, s);
         *launches += e == cudaSuccess;
         return e;
@@ -350,7 +337,7 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
         if (e != cudaSuccess) return e;
         ++*launches;
     }
-    if (odd && !A.last_as_block) {
+    if (odd) {
         if (tile_cut) slices_of(A, 0, A.n_chan, plan.tile_slices, part);
         else part[0] = A;
         e = launch_xeng_tile(part, tile_cut ? plan.tile_slices : 1, fresh && !tile_cut, zero_invalid, dev, status,
