@@ -177,10 +177,12 @@ int rounds_of(long long items, int workers) { return int((items + workers - 1) /
 // more rounds long integrations lose (512 x 152 x 6000, eight rounds, 333 -> 346 us): power
 // bounds them, and one kind's pairs end before the other's.  The last of an odd number of
 // tiles goes with the blocks, as one whose second tile is empty, where that takes no round
-// more (384 x 20 x 100, a launch less, 14.2 -> 12.4 us); where it does, only calls of one round
-// go in one launch, since its own launch then fills the pairs that a second round leaves idle
-// (384 x 52 x 5000 81 us, 99 with both kinds in one launch).
-constexpr int kBothRounds = 4;
+// more (384 x 20 x 100, a launch less, 14.2 -> 12.4 us).  Where it does, long integrations of
+// more than one round keep their launches, since the last tiles' then fills the pairs that the
+// last round leaves idle (384 x 52 x 5000 82 us, 104 with both kinds in one launch, 384 x 52 x
+// 1000 32.9 and 34.9); short ones gain all the same (384 x 76 x 100 26.7 -> 20.6 us, 640 x 36 x
+// 300 34.6 -> 27.8), except three rounds with a small last tile (272 x 98 x 300 28.8, 30.8).
+constexpr int kBothRounds = 4, kBothShortStages = 11;
 
 struct OneLaunch {
     bool fits = false, last_as_block = false;
@@ -202,7 +204,12 @@ OneLaunch one_launch(const TcArray &A, int sms)
     };
     if (rounds > kBothRounds) return l;
     l.last_as_block = tiles % 2 && divide(blocks + A.n_chan);
-    l.fits = l.last_as_block || (divide(blocks) && (tiles % 2 == 0 || rounds == 1));
+    if (l.last_as_block) {
+        l.fits = true;
+    } else if (divide(blocks)) {
+        const bool few = rounds == 2 || (rounds == 3 && A.n - 2 * kTile * half > kTile / 2);
+        l.fits = tiles % 2 == 0 || rounds == 1 || (few && A.nt <= 64 * kBothShortStages);
+    }
     return l;
 }
 

@@ -22,10 +22,11 @@ def test_last_tile_exact(N, F, T, zero_invalid):
     _check(N, F, T, zero_invalid)
 
 
-# one to four rounds of both kinds of items in one launch, one round with the last tiles apart, and
-# five rounds in launches of their own
+# one to four rounds of both kinds of items in one launch, one to three rounds with the last tiles
+# apart (short and longer integrations), and five rounds in launches of their own
 @pytest.mark.parametrize("N,F,T", [(512, 38, 70), (768, 20, 65), (1024, 14, 64), (400, 60, 63), (1024, 1, 200),
-                                   (640, 32, 130), (640, 12, 65), (500, 45, 64), (512, 95, 65)])
+                                   (640, 32, 130), (640, 12, 65), (500, 45, 64), (512, 95, 65), (384, 76, 65),
+                                   (384, 60, 705), (272, 98, 64), (380, 98, 63)])
 @pytest.mark.parametrize("zero_invalid", [False, True])
 def test_both_kinds_of_items_in_one_launch(N, F, T, zero_invalid):
     _check(N, F, T, zero_invalid)
