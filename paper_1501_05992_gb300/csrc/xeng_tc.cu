@@ -182,28 +182,29 @@ int rounds_of(long long items, int workers) { return int((items + workers - 1) /
 // last round leaves idle (384 x 52 x 5000 82 us, 104 with both kinds in one launch, 384 x 52 x
 // 1000 32.9 and 34.9); short ones gain all the same (384 x 76 x 100 26.7 -> 20.6 us, 640 x 36 x
 // 300 34.6 -> 27.8), except three rounds with a small last tile (272 x 98 x 300 28.8, 30.8).
+// In a call with others (alone = false) the last tiles go with theirs.
 constexpr int kBothRounds = 4, kBothShortStages = 11;
 
 struct OneLaunch {
     bool fits = false, last_as_block = false;
-    int block_pairs = 0, off_pairs = 0;
+    int rounds = 0, block_pairs = 0, off_pairs = 0;
 };
 
-OneLaunch one_launch(const TcArray &A, int sms)
+OneLaunch one_launch(const TcArray &A, int sms, bool alone)
 {
     OneLaunch l;
     const int tiles = tiles_of(A), half = tiles / 2, pairs = sms / 2;
     if (pairs < 2) return l;
     const long long blocks = (long long)A.n_chan * half,
                     offs = (long long)A.n_chan * (tiles % 2 ? half * half : half * (half - 1));
-    const int rounds = rounds_of(blocks + offs, pairs);
+    const int rounds = l.rounds = rounds_of(blocks + offs, pairs);
     auto divide = [&](long long with_blocks) {
         l.block_pairs = rounds_of(with_blocks, rounds);
         l.off_pairs = rounds_of(offs, rounds);
         return l.block_pairs + l.off_pairs <= pairs;
     };
     if (rounds > kBothRounds) return l;
-    l.last_as_block = tiles % 2 && divide(blocks + A.n_chan);
+    l.last_as_block = alone && tiles % 2 && divide(blocks + A.n_chan);
     if (l.last_as_block) {
         l.fits = true;
     } else if (divide(blocks)) {
@@ -237,7 +238,7 @@ LargePlan plan_large(const TcArray &A, int sms)
     if (pairs < 1) return plan;
     const int per_off = tiles % 2 ? half * half : half * (half - 1);
     const long long items = (long long)A.n_chan * (half + per_off);
-    const int lone = tiles % 2 && !one_launch(A, sms).last_as_block ? A.n_chan : 0;       // last tiles alone
+    const int lone = tiles % 2 && !one_launch(A, sms, true).last_as_block ? A.n_chan : 0;  // last tiles alone
     const int full = int(items / pairs), left = int(items % pairs);
     const int whole = rounds_of(items, pairs), idle = left ? sms - 2 * left : 0;
     // whole items; the last tiles take the SMs that the last round leaves idle first
@@ -295,6 +296,20 @@ __global__ void __launch_bounds__(256) zero_large_kernel(int2 *__restrict__ out,
     wait_for_launch_before();
 }
 
+// Both kinds of items of A in one launch; sets A.last_as_block.
+cudaError_t launch_one(TcArray &A, const OneLaunch &one, bool fresh, bool zero_invalid, int dev, DeviceStatus *status,
+                       const TcOptions &opt, cudaStream_t s, int *launches)
+{
+    A.last_as_block = one.last_as_block;
+    CUtensorMap map;
+    cudaError_t e = encode_map(A, &map);
+    if (e == cudaSuccess)
+        e = launch_xeng_both(A, map, one.block_pairs, one.off_pairs, fresh, zero_invalid, dev, status, opt,
+                             *launches > 0, s);
+    *launches += e == cudaSuccess;
+    return e;
+}
+
 // The launches of a call of one array of more than 256 inputs.
 cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, DeviceStatus *status, const TcOptions &opt,
                          cudaStream_t s, int *launches)
@@ -304,15 +319,9 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
     if (e != cudaSuccess) return e;
     const LargePlan plan = plan_large(A, sms);
     const bool odd = tiles_of(A) % 2, off_cut = plan.off_slices > 1, tile_cut = plan.tile_slices > 1;
-    const OneLaunch one = one_launch(A, sms);
+    const OneLaunch one = one_launch(A, sms, true);
     if (one.fits && !off_cut && !tile_cut) {
-        A.last_as_block = one.last_as_block;
-        CUtensorMap map;
-        e = encode_map(A, &map);
-        if (e == cudaSuccess)
-            e = launch_xeng_both(A, map, one.block_pairs, one.off_pairs, fresh, zero_invalid, dev, status, opt,
-                                 *launches > 0, s);
-        *launches += e == cudaSuccess;
+        e = launch_one(A, one, fresh, zero_invalid, dev, status, opt, s, launches);
         if (e != cudaSuccess || !odd || one.last_as_block) return e;
         e = launch_xeng_tile(&A, 1, fresh, zero_invalid, dev, status, opt, true, s);
         *launches += e == cudaSuccess;
@@ -354,6 +363,8 @@ cudaError_t launch_large(TcArray A, bool fresh, bool zero_invalid, int dev, Devi
     return e;
 }
 
+constexpr int kBothIdleStages = 16;
+
 // The launches of the arrays of one mode, longest integrations first (a CTA's
 // last items are then its shortest).
 // The launches of one call write disjoint parts of the output and may overlap: each lets
@@ -373,9 +384,32 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     cudaError_t e = cudaSuccess;
     if (count == 1 && m == 1 && sorted[0].n > 2 * kTile)
         return launch_large(sorted[0], fresh, zero_invalid, dev, status, opt, s, launches);
-    int n = 0;
+    // One array of more than 256 inputs beside some of up to 128 has both kinds of items in one
+    // launch, as one alone would, and the tiles take the SMs that it leaves: 512 and 128 inputs x
+    // 27 channels, two blocks of 168 samples 59.6 -> 54.0 us, 512 and 128 x 35, five of 349, 182
+    // -> 148, 512 x 23 x 312 and 128 x 26 x 433 24.6 -> 20.5.  Beside arrays of 129..256 inputs,
+    // whose blocks fill the pairs that the first launch leaves, it loses (512 and 192 x 26, five
+    // of 252, 133 -> 154); so do longer integrations of more than one round that leave over a
+    // quarter of the pairs idle (512 x 21 x 4509, 128 x 41 x 331 and 96 x 86 x 1971 74 -> 80).
+    int n = 0, apart = -1;
     for (int k = 0; k < m; ++k)
-        if (sorted[k].n > kTile) part[n++] = sorted[k];
+        if (sorted[k].n > kTile) apart = ++n == 1 && sorted[k].n > 2 * kTile ? k : -1;
+    if (apart >= 0) {
+        int sms = 0;
+        e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (e != cudaSuccess) return e;
+        const OneLaunch one = one_launch(sorted[apart], sms, false);
+        const bool full = one.rounds == 1 || 4 * (one.block_pairs + one.off_pairs) >= 3 * (sms / 2);
+        if (one.fits && (full || sorted[apart].nt <= 64 * kBothIdleStages)) {
+            e = launch_one(sorted[apart], one, fresh, zero_invalid, dev, status, opt, s, launches);
+            if (e != cudaSuccess) return e;
+        } else {
+            apart = -1;
+        }
+    }
+    n = 0;
+    for (int k = 0; k < m; ++k)
+        if (sorted[k].n > kTile && k != apart) part[n++] = sorted[k];
     // other launches of the call would fill the last round
     const bool alone = count == 1 && n == 1 && part[0].n <= 2 * kTile;
     if (n) e = launch_blocks(true, part, n, alone, fresh, zero_invalid, dev, status, opt, s, launches);
@@ -383,7 +417,7 @@ cudaError_t launch_group(const TcArray *arrays, int count, bool fresh, bool zero
     n = 0;
     CUtensorMap maps[kTcMaxArrays];
     for (int k = 0; k < m; ++k) {
-        if (sorted[k].n <= 2 * kTile) continue;
+        if (sorted[k].n <= 2 * kTile || k == apart) continue;
         e = encode_map(sorted[k], &maps[n]);
         if (e != cudaSuccess) return e;
         part[n++] = sorted[k];

@@ -42,6 +42,34 @@ def test_last_round_in_slices(N, F, T, zero_invalid):
     _check(N, F, T, zero_invalid)
 
 
+# (inputs, channels, samples) beside arrays of up to 128 inputs: one to four rounds of both kinds of
+# items, with last tiles and without, longer or shorter than the others' integrations; long ones that
+# leave pairs idle, and an array of 129..256 inputs beside, which keep their launches
+@pytest.mark.parametrize("arrays", [[(512, 27, 168), (128, 27, 168)], [(100, 30, 200), (320, 66, 130)],
+                                    [(384, 20, 65), (64, 200, 64), (128, 7, 300)], [(1024, 14, 64), (17, 5, 63)],
+                                    [(500, 21, 1025), (96, 40, 65)], [(512, 30, 1100), (128, 90, 64)],
+                                    [(128, 40, 130), (512, 38, 70), (256, 30, 100)], [(257, 9, 64), (384, 9, 130)]])
+@pytest.mark.parametrize("zero_invalid", [False, True])
+def test_large_array_beside_others(arrays, zero_invalid):
+    if not all(path_available("tc_fp8", n) for n, _, _ in arrays):
+        pytest.skip("tc_fp8 unsupported")
+    rng = np.random.default_rng(len(arrays) + arrays[0][1])
+    volts = [rng.integers(0, 256, (t, f, n), dtype=np.uint8) for n, f, t in arrays]
+    d = [torch.from_numpy(v).cuda() for v in volts]
+    b = corr.Batch([dict(n_inputs=n, n_chan=f, n_time_per_int=2 * t, path="tc_fp8", zero_invalid=zero_invalid)
+                    for n, f, t in arrays])
+    whole = b.integrate(d)
+    b.accumulate(d)
+    b.accumulate(d)
+    added = b.dump()
+    b.sync()
+    b.close()
+    for v, w, a in zip(volts, whole, added):
+        vis = oracle.xmac(v, zero_invalid)
+        assert np.array_equal(w.cpu().numpy(), oracle.to_int32(vis))
+        assert np.array_equal(a.cpu().numpy(), oracle.to_int32(2 * vis))
+
+
 def _check(N, F, T, zero_invalid):
     if not path_available("tc_fp8", N):
         pytest.skip("tc_fp8 unsupported")
